@@ -61,8 +61,10 @@ struct SpeciesDev {
   float dE_inv;
   int ntab;
   int nproc;
+  int charge;           // sign of q (FP64 comparisons are slow on this part)
   int heavy;            // samples the target neutral's velocity
   int np4;              // groups of four processes per table node: (nproc + 3) / 4
+  int pad;
   // cross sections (m^2) of all processes interleaved by node: entry
   // [node * np4 + g] holds processes 4g..4g+3 (zero past nproc)
   const float4* sig4;

@@ -8,6 +8,7 @@ namespace ecpic {
 
 constexpr int kPassBlock = 256;
 constexpr int kFieldBlock = 256;
+constexpr int kFieldOwners = 256;  // threads that scan a run's nodes (field_solve)
 constexpr int kCollideBlock = 256;
 
 struct BatchView {
@@ -48,6 +49,29 @@ void launch_pass(const BatchView& b, int grid, int mode, int only, cudaStream_t 
 void launch_collide(const BatchView& b, int grid, cudaStream_t s);
 void launch_field(const BatchView& b, int advance, int only, cudaStream_t s);
 void launch_phi(const BatchView& b, int slot, cudaStream_t s);
+
+// Several steps in one cooperative launch (steps.cu): each block works for
+// one run, blocks of the same run form its team.
+constexpr int kMaxStepBlocks = 160;
+struct StepTeams {
+  unsigned short slot[kMaxStepBlocks], index[kMaxStepBlocks], size[kMaxStepBlocks];
+  int blocks, threads;  // threads per block: 256 or 512
+};
+// Words of a run that its team shares, cleared before a launch.  births, imp
+// and fail rotate over three steps: one is added to, one is being read, one is
+// being cleared.
+struct __align__(128) StepWords {
+  unsigned arrive;  // arrivals at the team's barriers (a cache line of its own)
+  unsigned pad[31];
+  unsigned long long births[3][kMaxSpecies], imp[3][kMaxSpecies];
+  int fail[3];
+};
+struct StepPlan {
+  StepWords* words;             // max_slots
+  unsigned long long* deposit;  // per slot two more deposits, zero between launches
+};
+bool steps_fit(const BatchView& b, int device);
+cudaError_t launch_steps(const BatchView& b, const StepPlan& pl, const StepTeams& tm, int steps, cudaStream_t s);
 void launch_sort(const BatchView& b, int grid, cudaStream_t s);
 void launch_sort_phase(const BatchView& b, int grid, int phase, cudaStream_t s);
 void launch_init(const BatchView& b, int slot, const InitParams& p, cudaStream_t s);
@@ -65,6 +89,7 @@ void launch_deposit_device(int N, long long n, const int* cell, const float* xi,
 void launch_deposit2_device(int N, int periodic, long long n, const int* cell, const float* xi,
                             unsigned long long* S, cudaStream_t s);
 void read_checks(unsigned long long out[4]);
+void read_checks_steps(unsigned long long out[4]);
 void launch_philox_device(long long n, const uint32_t* ctr, const uint32_t* key, uint32_t* out,
                           cudaStream_t s);
 

@@ -161,6 +161,10 @@ class Batch {
   int choose_grid() const;
   bool stage_field(int grid) const;
   int step_chunk(long long n, std::string* err);
+  bool several_steps();
+  void form_teams();
+  size_t plan_deposit_bytes() const { return 2 * sizeof(unsigned long long) * (size_t)spc_ * (size_t)(nmax_ + 1); }
+  int step_several(long long n, std::string* err);
   // pinned host staging for uploads: a ring of kStageSlots buffers, each
   // reused once the copy recorded after its last use has left (an event);
   // nullptr (and *slot = -1) for larger images or without pinned memory
@@ -173,6 +177,7 @@ class Batch {
   // up to their end), to launch the rebalancing only where a run is due; the
   // kernels check the device state themselves
   bool rb_due_within(int steps) const;
+  int rb_first_due(int steps) const;  // steps to the first due run's level, at most `steps`
   void advance_levels(int steps);
   void rebalance_launch();
   int check(cudaError_t e, const char* what, std::string* err);
@@ -202,7 +207,12 @@ class Batch {
   uint8_t* d_rbmode_ = nullptr;
   int* d_rblist_ = nullptr;
   int* d_rbnum_ = nullptr;
+  StepTeams teams_{};
+  double fullest_ = 0.0;  // quads of the fullest block of teams_
+  bool teams_dirty_ = true;
+  StepPlan plan_{};  // of k_steps; null for a batch with more slots than blocks
   std::vector<long long> level_;  // predicted level of each slot
+  std::vector<long long> work_;   // its particles, as loaded or at the last growth check
   // runs admitted with defer, waiting for admit_wave()
   std::vector<int> wave_slots_;
   std::vector<InitParams> wave_params_;
