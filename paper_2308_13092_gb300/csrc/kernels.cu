@@ -37,11 +37,7 @@ __global__ void __launch_bounds__(kPassBlock, 4) k_pass(BatchView b, int mode, i
     Msm[2 * (b.nmax + 1) + i] = 0.0f;
   }
   if (threadIdx.x < kNumCtr) sh.ctr[threadIdx.x] = 0u;
-  if (threadIdx.x == 0) {
-    sh.lohi[0] = INT_MAX;
-    sh.lohi[1] = -1;
-    sh.nlive = 0u;
-  }
+  if (threadIdx.x == 0) sh.nlive = 0u;
   // the work is split in quads of particles, equal quads per CTA
   const long long T = seg_prefix(b, mode, only, pre, sh.wsm, 4);
   if (T == 0) return;
@@ -1163,7 +1159,7 @@ size_t pass_smem_bytes(const BatchView& b) {
   return sizeof(long long) * (size_t)(b.nseg + 1) +
          (b.weighted ? 4 : 3) * sizeof(uint32_t) * (size_t)(b.nmax + 1) +
          sizeof(float) * 3 * (size_t)(b.nmax + 1) +
-         sizeof(int) * (size_t)(3 * kRing) * (kPassBlock / 32) + sizeof(float) * (size_t)(b.nmax + 1);
+         sizeof(int) * (size_t)kRing * (kPassBlock / 32) + sizeof(float) * (size_t)(b.nmax + 1);
 }
 
 size_t field_smem_bytes(const BatchView& b) { return field_scratch_bytes(b.nmax, b.nseg / b.max_slots); }

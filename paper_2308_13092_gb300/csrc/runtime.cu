@@ -951,9 +951,13 @@ int Batch::choose_grid() const {
   const int occ = pass_max_ctas_per_sm(view());
   const long long cap = (long long)occ * sm_count_;
   long long want = (live_estimate() * 5 / 4 + kPassBlock * 2 - 1) / (kPassBlock * 2);
-  if (max_slots_ > 1) want = cap;  // a batch's population changes: fill the GPU
+  // a batch's population changes: fill the GPU, with two waves where a block of
+  // one would take 48 iterations or more (256 runs of 5e7 particles, 80
+  // iterations: 519 us per step with one wave, 508 with two; 64 runs of 1.2e7,
+  // 20 iterations: 168 and 172)
+  if (max_slots_ > 1) want = live_estimate() / 4 >= 48LL * kPassBlock * cap ? 2 * cap : cap;
   if (want < 1) want = 1;
-  return (int)std::min(cap, want);
+  return (int)(max_slots_ > 1 ? want : std::min(cap, want));
 }
 
 void Batch::invalidate_graphs() {

@@ -488,15 +488,16 @@ __device__ __forceinline__ void walk_nonuniform(int& c, float& f, float g, int N
   f = g;
 }
 
-constexpr int kRing = 160;  // candidate ring per warp: >= 31 left over + 4 * 32 added
+constexpr int kFarCell = -(1 << 30);
+constexpr int kRing = 160;  // candidates (indices) per warp: >= 31 left over + 4 * 32 added
 
 struct PassShared {
   uint32_t ctr[kNumCtr];  // this piece's counters (a piece has < 2^31 particles)
   uint32_t nlive;
   long long wsm[32];
   double dsm[32];
-  int lohi[2];
   unsigned top[2];  // k_steps: bounds of a sample's terms (zero between pieces)
+  int lowest;       // and the piece's lowest cell (INT_MAX)
 };
 
 // A run's step inside k_steps (shared memory): where the particles' phase
@@ -938,7 +939,7 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
   const SpeciesDev* SP = &R->sp[sp];
   const float qm_dt = SP->qm_dt, dtdx_u = R->dtdx_u;
   // the run's field staged in shared memory for the gather (after the rings)
-  float* Esm = reinterpret_cast<float*>(ring + sizeof(int) * (size_t)(3 * kRing) * (BLOCK / 32));
+  float* Esm = reinterpret_cast<float*>(ring + sizeof(int) * (size_t)kRing * (BLOCK / 32));
   // (launches whose CTAs take only an iteration or two read the field from
   // L1/L2 instead: the staging's barrier and round trip would not pay)
   if (STAGE) {
@@ -949,6 +950,8 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
   const float* E = FUSED ? field : STAGE ? Esm : R->E;
   const uint32_t thr24 = SP->thr24;
   const bool mcc = stepping && SP->nproc > 0 && thr24 > 0;
+  // (r0 >> 8) < thr24 as one comparison of r0
+  const uint32_t thr_last = (thr24 << 8) - 1u;  // 2^32 - 1 for thr24 = 2^24
   const bool heavy = SP->heavy != 0;
   const bool yz_stream = mcc && !heavy && thr24 >= (1u << 20);
   const bool load_yz = sample || yz_stream;
@@ -989,13 +992,13 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
     if (lane == 0) {
       atomicMax(&sh.top[0], eb);
       atomicMax(&sh.top[1], vb);
-      if (mom.w < N) atomicMin(&sh.lohi[0], lowest);
+      if (mom.w < N) atomicMin(&sh.lowest, lowest);
     }
     __syncthreads();
     em = __uint_as_float(sh.top[0]);
     vm = (__uint_as_float(sh.top[1]) + fabsf(qm_dt) * em) * 1.0001f;
     // (a margin for the cells that particles moved to since the sort)
-    if (mom.w < N) mom.w0 = max(0, min(N - mom.w, (sh.lohi[0] < N ? sh.lohi[0] : 0) - mom.w / 8));
+    if (mom.w < N) mom.w0 = max(0, min(N - mom.w, (sh.lowest < N ? sh.lowest : 0) - mom.w / 8));
     mom.e[0] = mom_bound(2.0f * vm * em * 1.0001f);
     mom.e[1] = mom_bound(vm);
     mom.e[2] = mom_bound(vm * vm * 1.0001f);
@@ -1005,21 +1008,22 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
     __syncthreads();
     if (threadIdx.x == 0) {
       sh.top[0] = sh.top[1] = 0u;
-      sh.lohi[0] = INT_MAX;
+      sh.lowest = INT_MAX;
     }
   }
 
-  int my_lo = INT_MAX, my_hi = -1;
   // kinetic energy of sample steps: each quad's four terms in FP32, the
   // quads summed in FP64 (one FP64 add per four particles: FP64 is slow on
   // this part), so the error per particle is a few FP32 roundings whatever
   // the number of particles a thread handles
   double ke = 0.0;
   unsigned ncand = 0, nlive = 0, nabs_l = 0, nabs_r = 0, nnan = 0, nimp_lost = 0;
-  // this warp's candidate ring: index, Philox word A.y, |g|^2 or vx
-  int* qi = reinterpret_cast<int*>(ring) + (threadIdx.x >> 5) * (3 * kRing);
-  uint32_t* qr = reinterpret_cast<uint32_t*>(qi + kRing);
-  float* qw = reinterpret_cast<float*>(qi + 2 * kRing);
+  // this warp's candidate ring: indices (the test reads the particle again and
+  // redraws its Philox block: about one particle in a hundred gets there)
+  int* qi = reinterpret_cast<int*>(ring) + (threadIdx.x >> 5) * kRing;
+  // a bound on the total collision rate per speed, squared, for the filter of
+  // the candidates (2^-16 covers every rounding of the comparison)
+  const float nu_max = SP->nu_max, nu_bnd2 = SP->nu_bnd * SP->nu_bnd * (1.0f + 1.0f / 65536.0f);
   int head = 0, wcount = 0;  // warp-uniform
   unsigned ncoll = 0;        // FUSED: lane p counts the collisions of process p
   uint32_t* dcnt = dep;
@@ -1094,9 +1098,17 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         }
       }
       bool cand[4] = {false, false, false, false};
-      bool hit[4] = {false, false, false, false};  // absorbed at x = 0 (impact tallies)
+      unsigned hit = 0u;  // bit j: absorbed at x = 0 (impact tallies)
+      if ((c[0] | c[1] | c[2] | c[3]) >= 0) {
+        nlive += 4u;
+      } else {
+        // absorbed particles: far from every cell, wherever the push takes them
 #pragma unroll
-      for (int j = 0; j < 4; ++j) nlive += c[j] >= 0 ? 1u : 0u;
+        for (int j = 0; j < 4; ++j) {
+          nlive += c[j] >= 0 ? 1u : 0u;
+          c[j] = c[j] >= 0 ? c[j] : kFarCell;
+        }
+      }
       if (stepping) {
         uint64_t id[4] = {0, 0, 0, 0};
         if (mcc) {
@@ -1130,9 +1142,8 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         float Ei[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const bool ok = c[j] >= 0 && chk(c[j] < N, 4, c[j], N);
-          if (!ok) c[j] = -1;
-          const int cc = ok ? c[j] : 0;
+          if (!chk(c[j] < N, 4, c[j], N)) c[j] = kFarCell;
+          const int cc = max(c[j], 0);
           if (scheme == ECPIC_SCHEME_EC) {
             Ei[j] = E[cc];
           } else if (order2 && scheme == ECPIC_SCHEME_MC2) {
@@ -1165,20 +1176,24 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
           }
         }
         float keq = 0.0f;
+        Float2 kef{0.0f, 0.0f};  // k_steps: the quad's terms without rounding their sum
         float pje[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const float vnew = v[j] + qm_dt * Ei[j];
           if (sample) {
             const float fk = weighted ? (float)kq[j] : 1.0f;
-            if (c[j] >= 0) keq += fk * (v[j] * vnew + yz[j]);
+            if (c[j] >= 0) {
+              if (FUSED) kef.add(fk * (v[j] * vnew + yz[j]));
+              else keq += fk * (v[j] * vnew + yz[j]);
+            }
             // J.E of the push, per cell at level k (scaled by q w / 2 dx later)
             pje[j] = c[j] >= 0 ? fk * ((v[j] + vnew) * Ei[j]) : 0.0f;
           }
           v[j] = vnew;
         }
         if (sample) {
-          ke += (double)keq;
+          ke += FUSED ? kef.value() : (double)keq;
           // J.E per cell of level k: per lane, then down each segment
           const int key = lane_cell_key(c);
           double* pwg = R->pw + (size_t)sp * N;
@@ -1231,39 +1246,76 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
           }
         }
         // Eq. 9 in cell units, then the walls: absorbed when X <= 0 or X >= L
+#pragma unroll
+        for (int j = 0; j < 4; ++j) cand[j] = mcc && r0[j] <= thr_last;
         if (uniform) {
+          int cj[4];
+          float g[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const bool live = c[j] >= 0;
-            const bool bad = live && !(fabsf(v[j]) < 3.0e8f);
-            float g = f[j] + v[j] * dtdx_u;
-            const float fl = floorf(g);
-            int cj = c[j] + (int)fl;
-            g -= fl;
-            const bool up = g >= 1.0f;  // g - floor(g) rounded to 1
-            cj += up ? 1 : 0;
-            g = up ? 0.0f : g;
-            if (!walls && (cj < 0 || cj >= N)) {
-              cj %= N;
-              if (cj < 0) cj += N;
+            g[j] = f[j] + v[j] * dtdx_u;
+            const float fl = floorf(g[j]);
+            cj[j] = c[j] + (int)fl;
+            g[j] -= fl;
+          }
+          // Nearly every quad stays inside: a live one with cells 0..N-1, off
+          // X = 0, offsets that did not round to 1 and finite speeds.  One set
+          // of tests per quad sees that (some tests wider than the rule); the
+          // others are told apart particle by particle in a rare branch.
+          const unsigned top = max(max((unsigned)cj[0], (unsigned)cj[1]), max((unsigned)cj[2], (unsigned)cj[3]));
+          const unsigned zero = min(min((unsigned)cj[0] | __float_as_uint(g[0]), (unsigned)cj[1] | __float_as_uint(g[1])),
+                                    min((unsigned)cj[2] | __float_as_uint(g[2]), (unsigned)cj[3] | __float_as_uint(g[3])));
+          const float gm = fmaxf(fmaxf(g[0], g[1]), fmaxf(g[2], g[3]));
+          const float vs = (fabsf(v[0]) + fabsf(v[1])) + (fabsf(v[2]) + fabsf(v[3]));
+          if (top < (unsigned)N && zero != 0u && gm < 1.0f && vs < 3.0e8f) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              c[j] = cj[j];
+              f[j] = g[j];
             }
-            const bool out = walls && (cj < 0 || cj >= N || (cj == 0 && g == 0.0f));
-            const bool ok = live && !bad && !out;
-            nnan += bad ? 1u : 0u;
-            nabs_r += (live && !bad && out && cj >= N) ? 1u : 0u;
-            nabs_l += (live && !bad && out && cj < N) ? 1u : 0u;
-            hit[j] = imp_on && live && !bad && out && cj < N;
-            c[j] = ok ? cj : -1;
-            f[j] = g;
-            cand[j] = mcc && ok && (r0[j] >> 8) < thr24;
+          } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              bool ok = c[j] >= 0;
+              if (ok) {
+                if (g[j] >= 1.0f) {  // g - floor(g) rounded to 1
+                  cj[j] += 1;
+                  g[j] = 0.0f;
+                }
+                if (!walls && (unsigned)cj[j] >= (unsigned)N) {
+                  cj[j] %= N;
+                  if (cj[j] < 0) cj[j] += N;
+                }
+                if (!(fabsf(v[j]) < 3.0e8f)) {
+                  ++nnan;
+                  ok = false;
+                } else if (walls && ((unsigned)cj[j] >= (unsigned)N || (cj[j] == 0 && g[j] == 0.0f))) {
+                  ok = false;
+                  if (cj[j] >= N) {
+                    ++nabs_r;
+                  } else {
+                    ++nabs_l;
+                    hit |= imp_on ? 1u << j : 0u;
+                  }
+                }
+              }
+              c[j] = ok ? cj[j] : -1;
+              f[j] = g[j];
+              cand[j] = cand[j] && ok;
+            }
           }
         } else {
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            if (c[j] < 0) continue;
+            if (c[j] < 0) {
+              c[j] = -1;
+              cand[j] = false;
+              continue;
+            }
             if (!(fabsf(v[j]) < 3.0e8f)) {
               ++nnan;
               c[j] = -1;
+              cand[j] = false;
               continue;
             }
             int cj = c[j];
@@ -1272,13 +1324,13 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
             if (walls && (cj < 0 || cj >= N || (cj == 0 && fj == 0.0f))) {
               nabs_r += cj >= N ? 1u : 0u;
               nabs_l += cj >= N ? 0u : 1u;
-              hit[j] = imp_on && cj < N;
+              hit |= imp_on && cj < N ? 1u << j : 0u;
               c[j] = -1;
+              cand[j] = false;
               continue;
             }
             c[j] = cj;
             f[j] = fj;
-            cand[j] = mcc && (r0[j] >> 8) < thr24;
           }
         }
         if (full) {
@@ -1296,17 +1348,17 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         }
         // ions absorbed at x = 0: their indices, for the impact tallies of the
         // collision kernel (the absorbed slot keeps its velocity until the sort)
-        if (imp_on && __any_sync(kFull, hit[0] || hit[1] || hit[2] || hit[3])) {
+        if (imp_on && __any_sync(kFull, hit != 0u)) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const unsigned m = __ballot_sync(kFull, hit[j]);
+            const unsigned m = __ballot_sync(kFull, (hit >> j) & 1u);
             if (m) {
               const int lead = __ffs(m) - 1;
               unsigned long long base = 0ull;
               if (lane == lead) base = atomicAdd(FUSED ? fx->imp + sp : (unsigned long long*)&ss->n_imp,
                                                   (unsigned long long)__popc(m));
               base = __shfl_sync(kFull, base, lead);
-              if (hit[j]) {
+              if ((hit >> j) & 1u) {
                 const long long idx = (long long)base + __popc(m & lt_mask);
                 if (idx >= G.imp_cap) ++nimp_lost;
                 else if (FUSED) tally_impact(b, s, slot, cur, (int)(i0 + j));
@@ -1327,28 +1379,28 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         if (mcc) {
           // a candidate with Rr >= nu_bnd |g| is a null collision whatever its
           // energy (the total rate never exceeds nu_bnd |g|): where |g| is at
-          // hand, only the others go on to the cross-section test
-          const float nu_max = SP->nu_max, nu_bnd = SP->nu_bnd;
+          // hand, only the others go on to the cross-section test.  Compared
+          // in squares, with Rr from 23 bits rounded down and the bound
+          // rounded up: the test itself decides what this lets through.
+          unsigned mine = 0u;
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const bool test = cand[j] && (!yz_stream ||
-                u24(ry[j]) * nu_max < nu_bnd * sqrtf(v[j] * v[j] + yz[j]));
             ncand += cand[j] ? 1u : 0u;
-            cand[j] = test;
+            const float Rl = (__uint_as_float((ry[j] >> 9) | 0x3F800000u) - 1.0f) * nu_max;
+            const bool null = yz_stream && Rl * Rl > nu_bnd2 * (v[j] * v[j] + yz[j]);
+            mine |= cand[j] && !null ? 1u << j : 0u;
           }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const unsigned m = __ballot_sync(kFull, cand[j]);
-            if (cand[j]) {
+          unsigned m = __ballot_sync(kFull, mine != 0u);
+          // one candidate per lane and round (mostly one round, or none)
+          while (m) {
+            if (mine) {
               int pos = head + wcount + __popc(m & lt_mask);
               if (pos >= kRing) pos -= kRing;
-              if (chk(pos >= 0 && pos < kRing, 5, pos, kRing)) {
-                qi[pos] = (int)(i0 + j);
-                qr[pos] = ry[j];
-                qw[pos] = yz_stream ? v[j] * v[j] + yz[j] : v[j];
-              }
+              if (chk(pos >= 0 && pos < kRing, 5, pos, kRing)) qi[pos] = (int)i0 + __ffs((int)mine) - 1;
+              mine &= mine - 1u;
             }
             wcount += __popc(m);
+            m = __ballot_sync(kFull, mine != 0u);
           }
         }
       }
@@ -1370,13 +1422,6 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
       }
       else
         dep_add4(dcnt, dlo, dhi, c, f);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (c[j] >= 0) {
-          my_lo = min(my_lo, c[j]);
-          my_hi = max(my_hi, c[j] + 1);
-        }
-      }
       if (sample) {
         // vx moments at the nodes of the new cell (CIC shares): per lane
         // summed where its particles share a cell, then down each segment
@@ -1491,35 +1536,31 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         int pos = head + lane;
         if (pos >= kRing) pos -= kRing;
         int i = 0;
-        uint32_t ryv = 0u;
-        float w = 0.0f;
+        uint64_t id = 0ull;
+        float vx = 0.0f, vy = 0.0f, vz = 0.0f, g2 = 0.0f, Rr = 0.0f;
         if (act) {
           i = qi[pos];
-          ryv = qr[pos];
-          w = qw[pos];
-        }
-        float g2 = w;
-        if (heavy) {
-          // relative speed to a target neutral drawn from the gas Maxwellian
-          if (act) {
-            const float vx = pvx[i], vy = pvy[i], vz = pvz[i];
-            const uint4 B = draw(seed, pid[i], (uint32_t)k, ((uint32_t)sp << 8) | 1u);
+          id = pid[i];
+          vx = pvx[i];
+          vy = pvy[i];
+          vz = pvz[i];
+          Rr = u24(draw(seed, id, (uint32_t)k, (uint32_t)sp << 8).y) * nu_max;
+          if (heavy) {
+            // relative speed to a target neutral drawn from the gas Maxwellian
+            const uint4 B = draw(seed, id, (uint32_t)k, ((uint32_t)sp << 8) | 1u);
             float z0, z1, z2, z3;
             box_muller(u24_open(B.x), u24(B.y), z0, z1);
             box_muller(u24_open(B.z), u24(B.w), z2, z3);
             const float sd = R->vth_gas;
             const float gx = vx - sd * z0, gy = vy - sd * z1, gz = vz - sd * z2;
             g2 = gx * gx + gy * gy + gz * gz;
-          }
-        } else if (!yz_stream) {
-          if (act) {
-            const float vy = pvy[i], vz = pvz[i];
-            g2 = w * w + (vy * vy + vz * vz);
+          } else if (yz_stream) {
+            g2 = vx * vx + yz2(vy, vz);
+          } else {
+            g2 = vx * vx + (vy * vy + vz * vz);
           }
         }
         const float gm = sqrtf(g2), En = SP->half_m_over_e * g2;
-        const float nu_max = SP->nu_max;
-        const float Rr = u24(ryv) * nu_max;
         float tot = 0.0f;
         int chosen = -1;
         if (act && Rr < SP->nu_bnd * gm) chosen = select_process(SP, En, gm, R->ng, Rr, &tot);
@@ -1533,14 +1574,14 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
             }
             if (chosen >= 0) {
               RealRec rec;
-              rec.id = pid[i];
+              rec.id = id;
               rec.i = i;
               rec.chosen = chosen;
               rec.En = En;
               rec.gm = gm;
-              rec.vx = pvx[i];
-              rec.vy = pvy[i];
-              rec.vz = pvz[i];
+              rec.vx = vx;
+              rec.vy = vy;
+              rec.vz = vz;
               rec.c = pc[i];
               rec.f = pxi[i];
               rec.k = weighted ? pwt[i] : 1u;
@@ -1557,12 +1598,10 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
           if (chosen >= 0) {
             const long long idx = (long long)base + __popc(m & lt_mask);
             if (idx < G.real_cap) {
-              const uint64_t id = pid[i];
               int4* dst = reinterpret_cast<int4*>(G.real + idx);  // RealRec field order
               dst[0] = make_int4((int)(uint32_t)id, (int)(uint32_t)(id >> 32), i, chosen);
-              dst[1] = make_int4(__float_as_int(En), __float_as_int(gm), __float_as_int(pvx[i]),
-                                 __float_as_int(pvy[i]));
-              dst[2] = make_int4(__float_as_int(pvz[i]), pc[i], __float_as_int(pxi[i]),
+              dst[1] = make_int4(__float_as_int(En), __float_as_int(gm), __float_as_int(vx), __float_as_int(vy));
+              dst[2] = make_int4(__float_as_int(vz), pc[i], __float_as_int(pxi[i]),
                                  weighted ? (int)pwt[i] : 1);
             } else {
               set_status(st, ECPIC_ERR_CAPACITY);
@@ -1630,9 +1669,7 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
     __syncthreads();
     return;
   }
-  // piece epilogue: node range, energy, counters, flush to HBM
-  my_lo = __reduce_min_sync(kFull, my_lo);
-  my_hi = __reduce_max_sync(kFull, my_hi);
+  // piece epilogue: energy, counters, flush to HBM
   ncand = __reduce_add_sync(kFull, ncand);
   nlive = __reduce_add_sync(kFull, nlive);
   nabs_l = __reduce_add_sync(kFull, nabs_l);
@@ -1641,10 +1678,6 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
   nimp_lost = __reduce_add_sync(kFull, nimp_lost);
   if (lane == 0) {
     if (stepping && nlive) atomicAdd(&sh.nlive, nlive);
-    if (my_hi >= 0) {
-      atomicMin(&sh.lohi[0], my_lo);
-      atomicMax(&sh.lohi[1], my_hi);
-    }
     if (ncand) atomicAdd(&sh.ctr[C_CAND], ncand);
     if (nabs_l) atomicAdd(&sh.ctr[C_ABS_L], nabs_l);
     if (nabs_r) atomicAdd(&sh.ctr[C_ABS_R], nabs_r);
@@ -1659,36 +1692,30 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
     if (threadIdx.x == 0) atomicAdd(&st->ke_acc[sp], 0.5 * SP->m * SP->w * kes);
   }
   __syncthreads();
-  const int flo = sh.lohi[0], fhi = chk(sh.lohi[1] <= N, 8, sh.lohi[1], N) ? sh.lohi[1] : N;
-  const int Nm = b.nmax + 1;
-  double* md = R->momd + (size_t)sp * 2 * (N + 1);
-  // an empty range (no live particle in the piece) is (INT_MAX, -1): skip it
-  // before forming flo + threadIdx.x, which would overflow
-  if (flo < fhi) {
-    if (order2)  // shares reach one node beyond the range, or wrap
-      dep2_flush(dlo, dhi, walls ? max(flo - 1, 0) : 0, walls ? min(fhi + 1, N) : N, Sg);
-    else if (weighted)
-      depw_flush(dw, flo, fhi, Sg);
-    else
-      dep_flush(dcnt, dlo, dhi, flo, fhi, Sg);
-  }
-  const int nbeg = flo <= fhi ? flo + (int)threadIdx.x : fhi + 1;
+  // (every cell: the range that the particles touch is not tracked, which
+  // costs the streaming loop more than the few reads of this scan)
+  if (order2)
+    dep2_flush(dlo, dhi, 0, N, Sg);
+  else if (weighted)
+    depw_flush(dw, 0, N, Sg);
+  else
+    dep_flush(dcnt, dlo, dhi, 0, N, Sg);
   if (sample) {
+    const int Nm = b.nmax + 1;
+    double* md = R->momd + (size_t)sp * 2 * (N + 1);
     double* pwg = R->pw + (size_t)sp * N;
-    for (int j = threadIdx.x; j < N; j += BLOCK) {
-      const float pj = Psm[j];
-      if (pj != 0.0f) {
-        atomicAdd(pwg + j, (double)pj);
-        Psm[j] = 0.0f;
+    for (int nn = threadIdx.x; nn <= N; nn += BLOCK) {
+      const float m1 = Msm[nn], m2 = Msm[Nm + nn];
+      if (m1 != 0.0f) atomicAdd(md + nn, (double)m1);
+      if (m2 != 0.0f) atomicAdd(md + (N + 1) + nn, (double)m2);
+      Msm[nn] = 0.0f;
+      Msm[Nm + nn] = 0.0f;
+      if (nn < N) {
+        const float pj = Psm[nn];
+        if (pj != 0.0f) atomicAdd(pwg + nn, (double)pj);
+        Psm[nn] = 0.0f;
       }
     }
-  }
-  for (int nn = nbeg; nn <= fhi && sample; nn += BLOCK) {
-    const float m1 = Msm[nn], m2 = Msm[Nm + nn];
-    if (m1 != 0.0f) atomicAdd(md + nn, (double)m1);
-    if (m2 != 0.0f) atomicAdd(md + (N + 1) + nn, (double)m2);
-    Msm[nn] = 0.0f;
-    Msm[Nm + nn] = 0.0f;
   }
   if (threadIdx.x < 32) {  // (kNumCtr < 32)
     const uint32_t val = lane < kNumCtr ? sh.ctr[lane] : lane == kNumCtr ? sh.nlive : 0u;
@@ -1704,11 +1731,6 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
     const uint32_t dead = __reduce_add_sync(
         kFull, lane == C_ABS_L || lane == C_ABS_R || lane == C_NAN ? val : 0u);
     if (lane == 0 && dead) atomicAdd((unsigned long long*)&ss->n_dead, (unsigned long long)dead);
-  }
-  __syncthreads();  // every thread has read the range
-  if (threadIdx.x == 0) {
-    sh.lohi[0] = INT_MAX;
-    sh.lohi[1] = -1;
   }
   __syncthreads();
 }

@@ -69,7 +69,7 @@ __host__ __device__ inline int scratch_words(int nmax, int species) {  // of 4 b
 __host__ __device__ inline size_t steps_bytes(int nmax, int species, bool weighted, int threads) {
   const size_t M = (size_t)nmax + 1;
   return kStepBase + M * (size_t)(3 * 8 + 4 + 4 * (weighted ? 4 : 3)) + 4 * (size_t)scratch_words(nmax, species) +
-         sizeof(int) * (size_t)(3 * kRing) * (size_t)(threads / 32);
+         sizeof(int) * (size_t)kRing * (size_t)(threads / 32);
 }
 
 // Where everything is.  Every function forms the addresses from the base of
@@ -212,8 +212,7 @@ __device__ __forceinline__ void step_piece(int s, long long k, unsigned beg, uns
   StepShared& sh = step_shared();
   const StepArrays a = step_arrays();
   const PieceState ps{sh.cur[s], sh.fx.n[s], k};
-  pass_piece<KIND, false, kStepBlock, true>(sh.b, &sh.run, sh.seg[s], sh.run.seg0 + s, ps, (long long)beg,
-                                            (long long)end, MODE_STEP, a.dep, a.mom, a.ring, sh.pass, &sh.fx, a.E,
+  pass_piece<KIND, false, kStepBlock, true>(sh.b, &sh.run, sh.seg[s], sh.run.seg0 + s, ps, (long long)beg, (long long)end, MODE_STEP, a.dep, a.mom, a.ring, sh.pass, &sh.fx, a.E,
                                             scratch_words(sh.b.nmax, sh.spc));
 }
 
@@ -536,7 +535,7 @@ __global__ void __launch_bounds__(kStepBlock, 1)
       sh.fx.fail = &words->fail[0];
       sh.fx.nlive = 0u;
       sh.pass.top[0] = sh.pass.top[1] = 0u;
-      sh.pass.lohi[0] = INT_MAX;
+      sh.pass.lowest = INT_MAX;
       split_team(sh, ns, team);
     }
     const StepArrays ar = step_arrays();
