@@ -18,11 +18,12 @@
 #include <mutex>
 
 #include "../../include/ecpic.h"
+#include "deposit.cuh"
 
 namespace {
 
 constexpr int kNaBlock = 256;
-constexpr int kNaMaxRows = 304;  // two blocks per SM on a 152-SM part
+constexpr int kNaMaxRows = 608;  // four blocks per SM on a 152-SM part
 constexpr size_t kNaWords = ECPIC_NOALLOC_SCRATCH_BYTES / sizeof(unsigned long long);
 constexpr int kMaxDevices = 64;
 
@@ -39,50 +40,79 @@ static __device__ __align__(256) unsigned long long g_na_scratch[kNaWords];
 std::mutex g_na_mu;
 void* g_na_ptr[kMaxDevices] = {};
 
-// Block-local deposit of a grid-stride share of the particles, written out
-// as this block's row.  Lanes holding the same cell add their shares once
-// (r = floor(xi * 2^32); the cell gets 2^32 - r, the next node r).
+// Block-local deposit of a block's consecutive quads, written out as this
+// block's row: 32-bit shared sums as in ecpic_deposit_device (deposit.cuh),
+// moved into 64-bit ones before they can overflow.  16.8 million particles on
+// 1024 cells with the sum of the rows: 61 us in cell order, 53 in random order
+// (64-bit shared atomics after a match of the lanes' cells: 340 and 990).
+template <bool VEC>
 __global__ void __launch_bounds__(kNaBlock) k_na_rows(int N, long long n, const int* __restrict__ cell,
                                                       const float* __restrict__ xi,
                                                       unsigned long long* rows) {
   extern __shared__ __align__(16) unsigned char na_smem[];
   unsigned long long* acc = reinterpret_cast<unsigned long long*>(na_smem);
-  for (int i = threadIdx.x; i <= N; i += kNaBlock) acc[i] = 0ull;
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  for (long long base = (long long)blockIdx.x * kNaBlock + (threadIdx.x & ~31); base < n;
-       base += (long long)gridDim.x * kNaBlock) {
-    const long long i = base + lane;
-    const int c = i < n ? cell[i] : -1;
-    const bool ok = c >= 0 && c < N;
-    const unsigned group = __match_any_sync(0xFFFFFFFFu, ok ? (unsigned)c : 0xFFFFFFFFu);
-    if (ok) {
-      const unsigned r = __float2uint_rz(xi[i] * 4294967296.0f);
-      // the 32-bit shares of up to 32 lanes, summed in two 16-bit halves
-      const unsigned lo = __reduce_add_sync(group, r & 0xFFFFu);
-      const unsigned hi = __reduce_add_sync(group, r >> 16);
-      if (lane == __ffs(group) - 1) {
-        const unsigned long long sr = ((unsigned long long)hi << 16) + lo;
-        const unsigned long long cnt = (unsigned long long)__popc(group);
-        atomicAdd(acc + c, (cnt << 32) - sr);
-        atomicAdd(acc + c + 1, sr);
-      }
-    }
+  uint32_t* dcnt = reinterpret_cast<uint32_t*>(acc + (N + 1));
+  uint32_t* dlo = dcnt + (N + 1);
+  uint32_t* dhi = dlo + (N + 1);
+  for (int i = threadIdx.x; i <= N; i += kNaBlock) {
+    acc[i] = 0ull;
+    dcnt[i] = dlo[i] = dhi[i] = 0u;
   }
   __syncthreads();
+  // node i takes 2^32 - r of its cell and r of the cell before
+  auto flush = [&]() {
+    __syncthreads();
+    for (int i = threadIdx.x; i <= N; i += kNaBlock) {
+      const unsigned long long own = ((unsigned long long)dhi[i] << 16) + dlo[i];
+      unsigned long long t = ((unsigned long long)dcnt[i] << 32) - own;
+      if (i > 0) t += ((unsigned long long)dhi[i - 1] << 16) + dlo[i - 1];
+      acc[i] += t;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i <= N; i += kNaBlock) dcnt[i] = dlo[i] = dhi[i] = 0u;
+    __syncthreads();
+  };
+  const long long nq = (n + 3) / 4;
+  const long long lo = nq * blockIdx.x / gridDim.x, hi = nq * (blockIdx.x + 1) / gridDim.x;
+  int since_flush = 0;
+  for (long long base = lo; base < hi; base += kNaBlock) {  // block-uniform trip count
+    const long long q = base + threadIdx.x;
+    int c[4];
+    float f[4];
+    ecpic::load_quad<VEC>(cell, xi, q < hi ? q : nq, n, N, c, f);
+    ecpic::dep_add_warp(dcnt, dlo, dhi, c, f);
+    if (++since_flush == ecpic::kFlushParticles / (4 * kNaBlock)) {
+      flush();
+      since_flush = 0;
+    }
+  }
+  flush();
   unsigned long long* row = rows + (size_t)blockIdx.x * (size_t)(N + 1);
   for (int i = threadIdx.x; i <= N; i += kNaBlock) row[i] = acc[i];
 }
 
-// S[i] += sum of the rows' entries i, in row order
+// S[i] += sum of the rows' entries i: a warp's lanes take 32 nodes, a block's
+// warps every kNaBlock / 32-th row (a serial sum over the rows by one thread
+// per node took longer than the rows of 10^5 particles)
 __global__ void __launch_bounds__(kNaBlock) k_na_sum(int N, int nrows,
                                                      const unsigned long long* __restrict__ rows,
                                                      unsigned long long* S) {
-  const int i = blockIdx.x * kNaBlock + threadIdx.x;
-  if (i > N) return;
+  constexpr int kWarps = kNaBlock / 32;
+  __shared__ unsigned long long part[kWarps][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
   unsigned long long s = 0ull;
-  for (int r = 0; r < nrows; ++r) s += rows[(size_t)r * (size_t)(N + 1) + i];
-  S[i] += s;
+  if (i <= N) {
+#pragma unroll 8
+    for (int r = w; r < nrows; r += kWarps) s += rows[(size_t)r * (size_t)(N + 1) + i];
+  }
+  part[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && i <= N) {
+#pragma unroll
+    for (int q = 1; q < kWarps; ++q) s += part[q][lane];
+    S[i] += s;
+  }
 }
 
 // The scratch address on the current device; the first call on a device
@@ -112,15 +142,18 @@ extern "C" int ecpic_deposit_device_noalloc(int N, int64_t n, const int32_t* d_c
   if (rc != ECPIC_OK) return rc;
   if (n == 0) return ECPIC_OK;
   const long long per_row = (long long)(kNaWords / (size_t)(N + 1));
-  long long nrows = (n + kNaBlock - 1) / kNaBlock;
+  long long nrows = (n + 8 * kNaBlock - 1) / (8 * kNaBlock);  // two iterations or more a block
   if (nrows > kNaMaxRows) nrows = kNaMaxRows;
   if (nrows > per_row) nrows = per_row;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // one row of N + 1 sums: at most 8 x 2049 = 16,392 B (N = 2048), within the
-  // 48 KiB a launch gets without an opt-in
-  const size_t smem = sizeof(unsigned long long) * (size_t)(N + 1);
-  k_na_rows<<<(unsigned)nrows, kNaBlock, smem, s>>>(N, (long long)n, d_cell, d_xi, rows);
-  k_na_sum<<<(unsigned)((N + 1 + kNaBlock - 1) / kNaBlock), kNaBlock, 0, s>>>(
+  // a row of N + 1 sums and three 32-bit ones per node: at most 20 x 2049 =
+  // 40,980 B (N = 2048), within the 48 KiB a launch gets without an opt-in
+  const size_t smem = (sizeof(unsigned long long) + 3 * sizeof(uint32_t)) * (size_t)(N + 1);
+  if (((reinterpret_cast<uintptr_t>(d_cell) | reinterpret_cast<uintptr_t>(d_xi)) & 15u) == 0u)
+    k_na_rows<true><<<(unsigned)nrows, kNaBlock, smem, s>>>(N, (long long)n, d_cell, d_xi, rows);
+  else
+    k_na_rows<false><<<(unsigned)nrows, kNaBlock, smem, s>>>(N, (long long)n, d_cell, d_xi, rows);
+  k_na_sum<<<(unsigned)((N + 1 + 31) / 32), kNaBlock, 0, s>>>(
       N, (int)nrows, rows, reinterpret_cast<unsigned long long*>(d_S));
   return cudaGetLastError() == cudaSuccess ? ECPIC_OK : ECPIC_ERR_CUDA;
 }

@@ -7,6 +7,7 @@
 #include <cfloat>
 #include <climits>
 
+#include "deposit.cuh"
 #include "kernels.h"
 
 namespace ecpic {
@@ -33,7 +34,6 @@ __device__ __noinline__ bool chk(bool ok, int where, long long idx, long long bo
 __device__ __forceinline__ bool chk(bool, int, long long, long long) { return true; }
 #endif
 
-constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr double kEps0 = 8.8541878128e-12;
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 
@@ -169,66 +169,6 @@ __device__ __forceinline__ int seg_find(const long long* pre, int nseg, long lon
 }
 
 // ----------------------------------------------------------------- deposit
-// Fixed-point CIC deposit (Eq. 2-3) in units of 2^-32 particle: a particle at
-// (c, xi) with r = floor(xi 2^32) (xi * 2^32 is exact in FP32; rz truncation
-// = floor) adds 2^32 - r to node c and r to node c+1.  In shared memory each
-// cell keeps three 32-bit sums, updated with native 32-bit atomics: its
-// particle count, and the sums of the low and high 16 bits of r.  The flush
-// forms the node values, S[c] += cnt 2^32 - R and S[c+1] += R with
-// R = hi 2^16 + lo.  With at most kFlushParticles particles between flushes
-// no sum reaches 2^32.
-constexpr int kFlushParticles = 65536;
-
-// Adds four particles (cells c[j] < 0 skipped); a thread's consecutive
-// particles in the same cell are merged first, so sorted data costs one
-// atomic triple per run.
-__device__ __forceinline__ void dep_add4(uint32_t* dcnt, uint32_t* dlo, uint32_t* dhi, const int c[4],
-                                         const float f[4]) {
-  unsigned lo[4], hi[4], cn[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const bool v = c[j] >= 0;
-    const unsigned r = v ? __float2uint_rz(f[j] * 4294967296.0f) : 0u;
-    lo[j] = r & 0xFFFFu;
-    hi[j] = r >> 16;
-    cn[j] = v ? 1u : 0u;
-  }
-#pragma unroll
-  for (int j = 3; j >= 1; --j) {
-    if (c[j] >= 0 && c[j] == c[j - 1]) {
-      lo[j - 1] += lo[j];
-      hi[j - 1] += hi[j];
-      cn[j - 1] += cn[j];
-      cn[j] = 0u;
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (cn[j]) {
-      atomicAdd(dcnt + c[j], cn[j]);
-      atomicAdd(dlo + c[j], lo[j]);
-      atomicAdd(dhi + c[j], hi[j]);
-    }
-  }
-}
-
-// Adds the shared sums of cells [a, e) to the node array S in HBM and clears
-// them.  Every thread of the block calls it, between barriers.
-__device__ void dep_flush(uint32_t* dcnt, uint32_t* dlo, uint32_t* dhi, int a, int e,
-                          unsigned long long* S) {
-  for (int c = a + (int)threadIdx.x; c < e; c += (int)blockDim.x) {
-    const uint32_t n = dcnt[c];
-    if (n) {
-      const unsigned long long R = ((unsigned long long)dhi[c] << 16) + (unsigned long long)dlo[c];
-      atomicAdd(S + c, ((unsigned long long)n << 32) - R);
-      if (R) atomicAdd(S + c + 1, R);
-      dcnt[c] = 0u;
-      dlo[c] = 0u;
-      dhi[c] = 0u;
-    }
-  }
-}
-
 // ---- weighted CIC deposit (rebalancing runs) -----------------------------
 // A particle of weight multiplier k adds k (2^32 - r) to node c and k r to
 // node c+1.  Shared 64-bit atomics are compare-and-swap loops on this part
@@ -292,85 +232,6 @@ __device__ void depw_flush(const DepW& d, int a, int e, unsigned long long* S) {
       d.a[c] = 0u;
       d.m[c] = 0u;
       d.b[c] = 0u;
-    }
-  }
-}
-
-// ---- quadratic-spline deposit of the EC2 scheme (uniform grids) ----------
-// A particle at cell + xi with r = floor(xi 2^32) has its nearest node
-// n0 = cell + (r >= 2^31) and offset U = r or r - 2^32 (2^-32 cell units);
-// nodes n0-1, n0, n0+1 get a = floor((2^31-U)^2 / 2^33), 2^32 - a - b,
-// b = floor((2^31+U)^2 / 2^33): the quadratic B-spline weights to 2^-32,
-// exact integers summing to 2^32.
-__device__ __forceinline__ void spline2_shares(float f, int c, int* n0, unsigned* a, unsigned* b) {
-  const unsigned r = __float2uint_rz(f * 4294967296.0f);
-  const bool up = r >= 0x80000000u;
-  *n0 = c + (up ? 1 : 0);
-  const long long U = up ? (long long)r - 4294967296LL : (long long)r;
-  const unsigned long long A = (unsigned long long)(2147483648LL - U);
-  const unsigned long long B = (unsigned long long)(2147483648LL + U);
-  *a = (unsigned)((__umul64hi(A, A) << 31) | ((A * A) >> 33));
-  *b = (unsigned)((__umul64hi(B, B) << 31) | ((B * B) >> 33));
-}
-
-// node of a share beyond the cells: folded into the wall node (Dirichlet: the
-// ghost node beyond a wall is the wall node), wrapped when periodic (node N
-// and node 0 are one node for the field solve)
-__device__ __forceinline__ int node2(int n, int N, bool periodic) {
-  if (periodic) return n < 0 ? n + N : (n > N ? n - N : n);
-  return n < 0 ? 0 : (n > N ? N : n);
-}
-
-// Adds four particles to two 32-bit sums per node (the low and high 16 bits
-// of the shares it receives, after folding or wrapping); runs of equal
-// nearest node merged first.  A wall node can receive two shares of one
-// particle, and a run's middle share can reach 2^34, so the EC2 pass flushes
-// every kFlushParticles / 4 particles: no sum reaches 2^32.
-__device__ __forceinline__ void dep2_add4(uint32_t* dlo, uint32_t* dhi, int N, bool periodic,
-                                          const int c[4], const float f[4]) {
-  int n0[4];
-  unsigned long long A[4], M[4], B[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    unsigned a = 0u, b = 0u;
-    n0[j] = -1;
-    if (c[j] >= 0) spline2_shares(f[j], c[j], &n0[j], &a, &b);
-    A[j] = a;
-    B[j] = b;
-    M[j] = c[j] >= 0 ? 4294967296ull - a - b : 0ull;
-  }
-#pragma unroll
-  for (int j = 3; j >= 1; --j) {
-    if (n0[j] >= 0 && n0[j] == n0[j - 1]) {
-      A[j - 1] += A[j];
-      M[j - 1] += M[j];
-      B[j - 1] += B[j];
-      n0[j] = -1;
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (n0[j] >= 0) {
-      const int nl = node2(n0[j] - 1, N, periodic), nr = node2(n0[j] + 1, N, periodic);
-      atomicAdd(dlo + nl, (unsigned)(A[j] & 0xFFFFu));
-      atomicAdd(dhi + nl, (unsigned)(A[j] >> 16));
-      atomicAdd(dlo + n0[j], (unsigned)(M[j] & 0xFFFFu));
-      atomicAdd(dhi + n0[j], (unsigned)(M[j] >> 16));
-      atomicAdd(dlo + nr, (unsigned)(B[j] & 0xFFFFu));
-      atomicAdd(dhi + nr, (unsigned)(B[j] >> 16));
-    }
-  }
-}
-
-// Adds the sums of nodes [a, e] to S and clears them; every thread of the
-// block calls it, between barriers.
-__device__ void dep2_flush(uint32_t* dlo, uint32_t* dhi, int a, int e, unsigned long long* S) {
-  for (int n = a + (int)threadIdx.x; n <= e; n += (int)blockDim.x) {
-    const unsigned long long v = ((unsigned long long)dhi[n] << 16) + dlo[n];
-    if (v) {
-      atomicAdd(S + n, v);
-      dlo[n] = 0u;
-      dhi[n] = 0u;
     }
   }
 }
