@@ -71,7 +71,9 @@ struct StepPlan {
   unsigned long long* deposit;  // per slot two more deposits, zero between launches
 };
 bool steps_fit(const BatchView& b, int device);
-cudaError_t launch_steps(const BatchView& b, const StepPlan& pl, const StepTeams& tm, int steps, cudaStream_t s);
+// sorts by cell after every sort_every-th step, since_sort steps after the last
+cudaError_t launch_steps(const BatchView& b, const StepPlan& pl, const StepTeams& tm, int steps, int sort_every,
+                         int since_sort, cudaStream_t s);
 void launch_sort(const BatchView& b, int grid, cudaStream_t s);
 void launch_sort_phase(const BatchView& b, int grid, int phase, cudaStream_t s);
 void launch_init(const BatchView& b, int slot, const InitParams& p, cudaStream_t s);

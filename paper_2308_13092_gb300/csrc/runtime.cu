@@ -23,6 +23,8 @@ constexpr size_t kAlign = 256;
 // 20.4 with 431, 26.1 against 23.7 with 862).
 constexpr double kStepQuads = 96.0;
 constexpr double kStepSmall = 400.0;
+// Steps of one launch of k_steps (a launch costs about 10 us).
+constexpr long long kStepsPerLaunch = 256;
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
@@ -1317,21 +1319,16 @@ bool Batch::several_steps() {
 
 int Batch::step_several(long long n, std::string* err) {
   const BatchView b = view();
-  const int sort_grid = choose_grid();
   while (n > 0) {
-    const int m = rb_first_due((int)std::min<long long>(n, sort_every_ - since_sort_));
-    int rc = check(launch_steps(b, plan_, teams_, m, stream_), "steps", err);
+    const int m = rb_first_due((int)std::min<long long>(n, kStepsPerLaunch));
+    int rc = check(launch_steps(b, plan_, teams_, m, sort_every_, since_sort_, stream_), "steps", err);
     if (rc) return rc;
     n -= m;
+    since_sort_ = (since_sort_ + m) % sort_every_;
     // the runs due at the new level rebalance (after its field)
     const bool due = rb_due_within(m);
     advance_levels(m);
     if (due) rebalance_launch();
-    since_sort_ += m;
-    if (since_sort_ >= sort_every_) {
-      launch_sort(b, sort_grid, stream_);
-      since_sort_ = 0;
-    }
   }
   return check(cudaGetLastError(), "step", err);
 }

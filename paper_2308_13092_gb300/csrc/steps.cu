@@ -44,7 +44,7 @@ struct StepShared {
   BatchView b;
   FusedStep fx;
   PassShared pass;
-  long long cap[kMaxSpecies];
+  long long cap[kMaxSpecies], fresh[kMaxSpecies];
   int cur[kMaxSpecies];
   unsigned first[kMaxSpecies + 1];  // the team's blocks of species s: first[s] .. first[s + 1] - 1
   unsigned long long wtot[kMaxSpecies][kStepWarps];
@@ -216,20 +216,28 @@ __device__ __forceinline__ void step_piece(int s, long long k, unsigned beg, uns
                                             scratch_words(sh.b.nmax, sh.spc));
 }
 
-// This block's share of its species' quads (of every species' where the team
-// is smaller than their number).
+// This block's share [beg, end) of species s's quads (every species has its
+// blocks; a team smaller than the number of species shares every species among
+// all its blocks).
+__device__ __forceinline__ bool step_share(const StepShared& sh, int s, unsigned me, unsigned team, unsigned* beg,
+                                           unsigned* end) {
+  const unsigned first = sh.split ? sh.first[s] : 0u;
+  const unsigned count = sh.split ? sh.first[s + 1] - first : team;
+  if (me < first || me - first >= count) return false;
+  const unsigned T = (unsigned)((sh.fx.n[s] + 3) >> 2);
+  const unsigned per = (T + count - 1) / count;
+  *beg = min(T, per * (me - first));
+  *end = min(T, *beg + per);
+  return *beg < *end;
+}
+
 template <bool WEIGHTED, int kStepBlock>
 __device__ __forceinline__ void step_particles(unsigned me, unsigned team, long long k, bool sample) {
   const StepShared& sh = step_shared();
   const int ns = sh.run.ns;
   for (int s = 0; s < ns; ++s) {
-    const unsigned first = sh.split ? sh.first[s] : 0u;
-    const unsigned count = sh.split ? sh.first[s + 1] - first : team;
-    if (me < first || me - first >= count) continue;
-    const unsigned T = (unsigned)((sh.fx.n[s] + 3) >> 2);
-    const unsigned per = (T + count - 1) / count;
-    const unsigned beg = min(T, per * (me - first)), end = min(T, beg + per);
-    if (beg >= end) continue;
+    unsigned beg, end;
+    if (!step_share(sh, s, me, team, &beg, &end)) continue;
     if (sh.run.scheme >= ECPIC_SCHEME_EC2)
       step_piece<2, kStepBlock>(s, k, beg, end);
     else if (WEIGHTED && sh.run.rb && sample)
@@ -240,6 +248,120 @@ __device__ __forceinline__ void step_particles(unsigned me, unsigned team, long 
       step_piece<1, kStepBlock>(s, k, beg, end);
     else
       step_piece<0, kStepBlock>(s, k, beg, end);
+  }
+}
+
+// ---- counting sort by cell, between the barriers of a team -----------------
+// The cells of a block's share of each species: counted in H (shared memory,
+// one array per species, kept for the scatter) and added to the run's
+// histogram.
+template <int kStepBlock>
+__device__ __noinline__ void sort_count(unsigned me, unsigned team) {
+  const StepShared& sh = step_shared();
+  const int ns = sh.run.ns, N = sh.run.N, M = N + 1;
+  int* H = reinterpret_cast<int*>(step_arrays().mom);
+  for (int i = threadIdx.x; i < ns * M; i += kStepBlock) H[i] = 0;
+  __syncthreads();
+  for (int s = 0; s < ns; ++s) {
+    unsigned beg, end;
+    if (!step_share(sh, s, me, team, &beg, &end)) continue;
+    const int32_t* pc = sh.seg[s].cell[sh.cur[s]];
+    const long long n = sh.fx.n[s];
+    int* h = H + s * M;
+    for (unsigned q = beg + threadIdx.x; q < end; q += kStepBlock) {
+      int at = -1, run = 0;  // runs of equal cells, one atomic each
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const long long i = 4ll * q + j;
+        const int c = i < n ? pc[i] : -1;
+        if (c != at) {
+          if (at >= 0) atomicAdd(h + at, run);
+          at = c;
+          run = 0;
+        }
+        ++run;
+      }
+      if (at >= 0) atomicAdd(h + at, run);
+    }
+  }
+  __syncthreads();
+  for (int s = 0; s < ns; ++s)
+    for (int c = threadIdx.x; c < N; c += kStepBlock)
+      if (H[s * M + c]) atomicAdd(sh.b.hist + sh.seg[s].hoff + c, H[s * M + c]);
+}
+
+// The share's particles to their cells' places in the other buffer set: a cell
+// starts at the prefix of the histogram, a block reserves its part of it with
+// one atomic.  fresh[s]: the species' particles after the sort.
+template <int kStepBlock>
+__device__ __noinline__ void sort_scatter(unsigned me, unsigned team, long long* fresh) {
+  StepShared& sh = step_shared();
+  const int ns = sh.run.ns, N = sh.run.N, M = N + 1, tid = threadIdx.x;
+  int* H = reinterpret_cast<int*>(step_arrays().mom);
+  const int per = (N + kStepBlock - 1) / kStepBlock;
+  const int cb = min(N, tid * per), ce = min(N, cb + per);
+  for (int s = 0; s < ns; ++s) {
+    const int* hist = sh.b.hist + sh.seg[s].hoff;
+    int* taken = sh.b.rbcnt + sh.seg[s].hoff;
+    int loc = 0, total;
+    for (int c = cb; c < ce; ++c) loc += hist[c];
+    int at = block_excl_scan(loc, reinterpret_cast<int*>(sh.wsm), &total);
+    if (tid == 0) fresh[s] = total;
+    for (int c = cb; c < ce; ++c) {
+      const int mine = H[s * M + c], all = hist[c];
+      if (mine) H[s * M + c] = at + atomicAdd(taken + c, mine);
+      at += all;
+    }
+  }
+  __syncthreads();
+  for (int s = 0; s < ns; ++s) {
+    unsigned beg, end;
+    if (!step_share(sh, s, me, team, &beg, &end)) continue;
+    const SegDev& G = sh.seg[s];
+    const int a = sh.cur[s], o = a ^ 1;
+    const long long n = sh.fx.n[s];
+    int* h = H + s * M;
+    for (unsigned q = beg + tid; q < end; q += kStepBlock) {
+      int c[4], d[4];
+      float x[4], u[4], v[4], w[4];
+      uint64_t id[4];
+      unsigned kw[4] = {1u, 1u, 1u, 1u};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const long long i = 4ll * q + j;
+        c[j] = i < n ? G.cell[a][i] : -1;
+        const bool in = c[j] >= 0;
+        x[j] = in ? G.xi[a][i] : 0.0f;
+        u[j] = in ? G.vx[a][i] : 0.0f;
+        v[j] = in ? G.vy[a][i] : 0.0f;
+        w[j] = in ? G.vz[a][i] : 0.0f;
+        id[j] = in ? G.id[a][i] : 0ull;
+        if (in && G.wt[a]) kw[j] = G.wt[a][i];
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        // a run of equal cells takes its places with one atomic
+        const bool head = j == 0 || c[j] != c[j - 1];
+        int run = 1;
+        if (head)
+          for (int l = j + 1; l < 4; ++l) {
+            if (c[l] != c[j]) break;
+            ++run;
+          }
+        d[j] = c[j] < 0 ? -1 : head ? atomicAdd(h + c[j], run) : d[j - 1] + 1;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (d[j] < 0 || !chk(d[j] < G.cap, 35, d[j], G.cap)) continue;
+        G.cell[o][d[j]] = c[j];
+        G.xi[o][d[j]] = x[j];
+        G.vx[o][d[j]] = u[j];
+        G.vy[o][d[j]] = v[j];
+        G.vz[o][d[j]] = w[j];
+        G.id[o][d[j]] = id[j];
+        if (G.wt[o]) G.wt[o][d[j]] = kw[j];
+      }
+    }
   }
 }
 
@@ -489,7 +611,8 @@ __device__ __noinline__ void step_field(const unsigned long long* S, double phi0
 
 template <bool WEIGHTED, int kStepBlock>
 __global__ void __launch_bounds__(kStepBlock, 1)
-    k_steps(BatchView gb, StepPlan pl, __grid_constant__ const StepTeams tm, int steps) {
+    k_steps(BatchView gb, StepPlan pl, __grid_constant__ const StepTeams tm, int steps, int sort_every,
+            int since_sort) {
   StepShared& sh = step_shared();
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int slot = tm.slot[blockIdx.x];
@@ -569,9 +692,10 @@ __global__ void __launch_bounds__(kStepBlock, 1)
     __syncthreads();
     if (tid == 0) arrive(&words->arrive);
     arrivals += team;
+    const bool sort = since_sort + 1 == sort_every;
     // the first block of the team closes the launch (the others help with its
-    // sample)
-    if (last && me != 0 && !sample) break;
+    // sample and its sort)
+    if (last && me != 0 && !sample && !sort) break;
     const double phi0 = sh.phi0[t & 31];
     if (!await(&words->arrive, arrivals, sh)) {
       if (tid == 0) set_status(st, ECPIC_ERR_TIMEOUT);
@@ -625,9 +749,44 @@ __global__ void __launch_bounds__(kStepBlock, 1)
       if (tid < ns) sst[tid].n_proc = sst[tid].n_alloc = sh.fx.n[tid];
     }
     __syncthreads();
+    since_sort = sort ? 0 : since_sort + 1;
+    if (sort) {
+      flush_counters<kStepBlock>(sh, st, sst, ns);  // (the sort ends the count of absorbed slots)
+      __syncthreads();
+      sort_count<kStepBlock>(me, team);
+      __syncthreads();
+      if (tid == 0) arrive(&words->arrive);
+      arrivals += team;
+      bool ok = await(&words->arrive, arrivals, sh);
+      if (ok) {
+        sort_scatter<kStepBlock>(me, team, sh.fresh);
+        __syncthreads();
+        if (tid == 0) arrive(&words->arrive);
+        arrivals += team;
+        ok = await(&words->arrive, arrivals, sh);
+      }
+      if (!ok) {
+        if (tid == 0) set_status(st, ECPIC_ERR_TIMEOUT);
+        break;
+      }
+      // the run's cell arrays end at zero
+      for (int s = 0; s < ns; ++s)
+        for (int c = tid + kStepBlock * (int)me; c < N; c += kStepBlock * (int)team)
+          gb.hist[sh.seg[s].hoff + c] = gb.rbcnt[sh.seg[s].hoff + c] = 0;
+      if (tid < ns) {
+        sh.cur[tid] ^= 1;
+        sh.fx.n[tid] = sh.fresh[tid];
+        if (me == 0) {
+          sst[tid].cur = sh.cur[tid];
+          sst[tid].n_proc = sst[tid].n_alloc = sst[tid].n_live = sh.fresh[tid];
+          sst[tid].n_dead = 0;
+        }
+      }
+      __syncthreads();
+    }
     if (last) {
       // every deposit ends at zero, this step's once all have read it
-      if (sample) {
+      if (sample && !sort) {
         if (me != 0) {
           if (tid == 0) arrive(&words->arrive);
           break;
@@ -637,7 +796,8 @@ __global__ void __launch_bounds__(kStepBlock, 1)
           break;
         }
       }
-      for (int i = tid; i < ns * M; i += kStepBlock) S[i] = Sz[i] = 0ull;
+      if (me == 0)
+        for (int i = tid; i < ns * M; i += kStepBlock) S[i] = Sz[i] = 0ull;
       break;
     }
     if (sample && se == 1) {
@@ -667,7 +827,8 @@ size_t steps_smem(const BatchView& b, int threads) {
 }
 
 template <bool W, int kStepBlock>
-cudaError_t launch_w(const BatchView& b, const StepPlan& pl, const StepTeams& tm, int steps, cudaStream_t s) {
+cudaError_t launch_w(const BatchView& b, const StepPlan& pl, const StepTeams& tm, int steps, int sort_every,
+                     int since_sort, cudaStream_t s) {
   const size_t sm = steps_smem(b, kStepBlock);
   cudaError_t e = cudaFuncSetAttribute(k_steps<W, kStepBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
@@ -681,7 +842,7 @@ cudaError_t launch_w(const BatchView& b, const StepPlan& pl, const StepTeams& tm
   at.val.cooperative = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_steps<W, kStepBlock>, b, pl, tm, steps);
+  return cudaLaunchKernelEx(&cfg, k_steps<W, kStepBlock>, b, pl, tm, steps, sort_every, since_sort);
 }
 
 }  // namespace
@@ -693,12 +854,15 @@ bool steps_fit(const BatchView& b, int device) {
   return coop != 0 && steps_smem(b, 512) + 1024 <= (size_t)most;
 }
 
-cudaError_t launch_steps(const BatchView& b, const StepPlan& pl, const StepTeams& tm, int steps, cudaStream_t s) {
+cudaError_t launch_steps(const BatchView& b, const StepPlan& pl, const StepTeams& tm, int steps, int sort_every,
+                         int since_sort, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(pl.words, 0, sizeof(StepWords) * (size_t)b.max_slots, s);
   if (e != cudaSuccess) return e;
   if (tm.threads == 256)
-    return b.weighted ? launch_w<true, 256>(b, pl, tm, steps, s) : launch_w<false, 256>(b, pl, tm, steps, s);
-  return b.weighted ? launch_w<true, 512>(b, pl, tm, steps, s) : launch_w<false, 512>(b, pl, tm, steps, s);
+    return b.weighted ? launch_w<true, 256>(b, pl, tm, steps, sort_every, since_sort, s)
+                      : launch_w<false, 256>(b, pl, tm, steps, sort_every, since_sort, s);
+  return b.weighted ? launch_w<true, 512>(b, pl, tm, steps, sort_every, since_sort, s)
+                    : launch_w<false, 512>(b, pl, tm, steps, sort_every, since_sort, s);
 }
 
 void read_checks_steps(unsigned long long out[4]) {
