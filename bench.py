@@ -83,7 +83,7 @@ def kernel_code(text):
 def kernel_sources_sha256():
     import hashlib
     h = hashlib.sha256()
-    for f in ("kernels.cu", "step_dev.cuh", "ecpic_dev.cuh"):
+    for f in ("kernels.cu", "step_dev.cuh", "deposit.cuh", "ecpic_dev.cuh"):
         with open(os.path.join(ROOT, "paper_2308_13092_gb300", "csrc", f), encoding="utf-8") as fh:
             h.update(kernel_code(fh.read()).encode())
     return h.hexdigest()

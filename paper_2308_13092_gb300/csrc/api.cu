@@ -538,6 +538,7 @@ int ecpic_debug_checks(int64_t* out) {
   unsigned long long v[4] = {0, 0, 0, 0};
   ecpic::read_checks(v);
   if (v[3] == 0) ecpic::read_checks_steps(v);
+  if (v[3] == 0) ecpic::read_checks_steps_weighted(v);
   for (int i = 0; i < 4; ++i) out[i] = (int64_t)v[i];
   return cudaGetLastError() == cudaSuccess ? ECPIC_OK : ECPIC_ERR_CUDA;
 }

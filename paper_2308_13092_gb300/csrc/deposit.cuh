@@ -21,14 +21,15 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // no sum reaches 2^32.
 constexpr int kFlushParticles = 65536;
 
-// Adds four particles (cells c[j] < 0 skipped); a thread's consecutive
+// Adds V particles (cells c[j] < 0 skipped); a thread's consecutive
 // particles in the same cell are merged first, so sorted data costs one
 // atomic triple per run.
-__device__ __forceinline__ void dep_add4(uint32_t* dcnt, uint32_t* dlo, uint32_t* dhi, const int c[4],
-                                         const float f[4]) {
-  unsigned lo[4], hi[4], cn[4];
+template <int V = 4>
+__device__ __forceinline__ void dep_add4(uint32_t* dcnt, uint32_t* dlo, uint32_t* dhi, const int c[V],
+                                         const float f[V]) {
+  unsigned lo[V], hi[V], cn[V];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < V; ++j) {
     const bool v = c[j] >= 0;
     const unsigned r = v ? __float2uint_rz(f[j] * 4294967296.0f) : 0u;
     lo[j] = r & 0xFFFFu;
@@ -36,7 +37,7 @@ __device__ __forceinline__ void dep_add4(uint32_t* dcnt, uint32_t* dlo, uint32_t
     cn[j] = v ? 1u : 0u;
   }
 #pragma unroll
-  for (int j = 3; j >= 1; --j) {
+  for (int j = V - 1; j >= 1; --j) {
     if (c[j] >= 0 && c[j] == c[j - 1]) {
       lo[j - 1] += lo[j];
       hi[j - 1] += hi[j];
@@ -45,7 +46,7 @@ __device__ __forceinline__ void dep_add4(uint32_t* dcnt, uint32_t* dlo, uint32_t
     }
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < V; ++j) {
     if (cn[j]) {
       atomicAdd(dcnt + c[j], cn[j]);
       atomicAdd(dlo + c[j], lo[j]);
@@ -96,17 +97,18 @@ __device__ __forceinline__ int node2(int n, int N, bool periodic) {
   return n < 0 ? 0 : (n > N ? N : n);
 }
 
-// Adds four particles to two 32-bit sums per node (the low and high 16 bits
+// Adds V particles to two 32-bit sums per node (the low and high 16 bits
 // of the shares it receives, after folding or wrapping); runs of equal
 // nearest node merged first.  A wall node can receive two shares of one
 // particle, and a run's middle share can reach 2^34, so the EC2 pass flushes
 // every kFlushParticles / 4 particles: no sum reaches 2^32.
+template <int V = 4>
 __device__ __forceinline__ void dep2_add4(uint32_t* dlo, uint32_t* dhi, int N, bool periodic,
-                                          const int c[4], const float f[4]) {
-  int n0[4];
-  unsigned long long A[4], M[4], B[4];
+                                          const int c[V], const float f[V]) {
+  int n0[V];
+  unsigned long long A[V], M[V], B[V];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < V; ++j) {
     unsigned a = 0u, b = 0u;
     n0[j] = -1;
     if (c[j] >= 0) spline2_shares(f[j], c[j], &n0[j], &a, &b);
@@ -115,7 +117,7 @@ __device__ __forceinline__ void dep2_add4(uint32_t* dlo, uint32_t* dhi, int N, b
     M[j] = c[j] >= 0 ? 4294967296ull - a - b : 0ull;
   }
 #pragma unroll
-  for (int j = 3; j >= 1; --j) {
+  for (int j = V - 1; j >= 1; --j) {
     if (n0[j] >= 0 && n0[j] == n0[j - 1]) {
       A[j - 1] += A[j];
       M[j - 1] += M[j];
@@ -124,7 +126,7 @@ __device__ __forceinline__ void dep2_add4(uint32_t* dlo, uint32_t* dhi, int N, b
     }
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < V; ++j) {
     if (n0[j] >= 0) {
       const int nl = node2(n0[j] - 1, N, periodic), nr = node2(n0[j] + 1, N, periodic);
       atomicAdd(dlo + nl, (unsigned)(A[j] & 0xFFFFu));

@@ -56,6 +56,7 @@ constexpr int kMaxStepBlocks = 160;
 struct StepTeams {
   unsigned short slot[kMaxStepBlocks], index[kMaxStepBlocks], size[kMaxStepBlocks];
   int blocks, threads;  // threads per block: 256 or 512
+  int group;            // consecutive particles per thread: 1, 2 or 4
 };
 // Words of a run that its team shares, cleared before a launch.  births, imp
 // and fail rotate over three steps: one is added to, one is being read, one is
@@ -74,6 +75,8 @@ bool steps_fit(const BatchView& b, int device);
 // sorts by cell after every sort_every-th step, since_sort steps after the last
 cudaError_t launch_steps(const BatchView& b, const StepPlan& pl, const StepTeams& tm, int steps, int sort_every,
                          int since_sort, cudaStream_t s);
+cudaError_t launch_steps_weighted(const BatchView& b, const StepPlan& pl, const StepTeams& tm, int steps,
+                                  int sort_every, int since_sort, cudaStream_t s);
 void launch_sort(const BatchView& b, int grid, cudaStream_t s);
 void launch_sort_phase(const BatchView& b, int grid, int phase, cudaStream_t s);
 void launch_init(const BatchView& b, int slot, const InitParams& p, cudaStream_t s);
@@ -92,6 +95,7 @@ void launch_deposit2_device(int N, int periodic, long long n, const int* cell, c
                             unsigned long long* S, cudaStream_t s);
 void read_checks(unsigned long long out[4]);
 void read_checks_steps(unsigned long long out[4]);
+void read_checks_steps_weighted(unsigned long long out[4]);
 void launch_philox_device(long long n, const uint32_t* ctr, const uint32_t* key, uint32_t* out,
                           cudaStream_t s);
 

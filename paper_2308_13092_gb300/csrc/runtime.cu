@@ -16,13 +16,18 @@ namespace {
 constexpr double kQe = 1.602176634e-19;
 constexpr double kKb = 1.380649e-23;
 constexpr size_t kAlign = 256;
-// Quads of particles per block of k_steps below which more blocks do not pay
-// (16,384 particles on 42 blocks: 1.5 us per step less than on 16), and up to
-// which 256 threads with 255 registers beat 512 with 128 (us per step, without
-// samples and sorts: 12.1 against 13.6 with 96 quads per block, 20.6 against
-// 20.4 with 431, 26.1 against 23.7 with 862).
-constexpr double kStepQuads = 96.0;
+// Quads of particles per block of k_steps below which more blocks do not pay,
+// and up to which 256 threads with 255 registers beat 512 with 128 (us per
+// step, without samples and sorts: 12.1 against 13.6 with 96 quads per block,
+// 20.6 against 20.4 with 431, 26.1 against 23.7 with 862).
+constexpr double kStepQuads = 48.0;
 constexpr double kStepSmall = 400.0;
+// Particles of the fullest block up to which a thread takes one or two of them
+// at a time instead of four: a block's time is then the chain of one warp's
+// instructions, which are fewer (us per step: 16,384 particles, 195 per block,
+// 12.2 with one, 12.7 with two, 13.1 with four; 58,254, 383 per block, 12.7,
+// 12.2 and 13.3; 131,072, 862 per block, 13.8 with two, 13.2 with four).
+constexpr double kStepOne = 256.0, kStepTwo = 512.0;
 // Steps of one launch of k_steps (a launch costs about 10 us).
 constexpr long long kStepsPerLaunch = 256;
 
@@ -1295,6 +1300,7 @@ void Batch::form_teams() {
     }
   }
   teams_.threads = fullest_ <= kStepSmall ? 256 : 512;
+  teams_.group = 4.0 * fullest_ <= kStepOne ? 1 : 4.0 * fullest_ <= kStepTwo ? 2 : 4;
 }
 
 // Whether the batch advances by k_steps.  Its step takes the time of its

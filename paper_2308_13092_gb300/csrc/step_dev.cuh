@@ -183,11 +183,12 @@ struct DepW {
   uint32_t *k, *a, *m, *b;  // (nmax + 1) each
 };
 
-__device__ __forceinline__ void depw_add4(const DepW& d, const int c[4], const float f[4],
-                                          const unsigned kq[4]) {
-  unsigned K[4], A[4], M[4], B[4];
+template <int V = 4>
+__device__ __forceinline__ void depw_add4(const DepW& d, const int c[V], const float f[V],
+                                          const unsigned kq[V]) {
+  unsigned K[V], A[V], M[V], B[V];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < V; ++j) {
     const bool v = c[j] >= 0;
     const unsigned r = v ? __float2uint_rz(f[j] * 4294967296.0f) : 0u;
     const unsigned k = v ? kq[j] : 0u;
@@ -198,7 +199,7 @@ __device__ __forceinline__ void depw_add4(const DepW& d, const int c[4], const f
     B[j] = q >> 16;
   }
 #pragma unroll
-  for (int j = 3; j >= 1; --j) {
+  for (int j = V - 1; j >= 1; --j) {
     if (c[j] >= 0 && c[j] == c[j - 1]) {
       K[j - 1] += K[j];
       A[j - 1] += A[j];
@@ -208,7 +209,7 @@ __device__ __forceinline__ void depw_add4(const DepW& d, const int c[4], const f
     }
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < V; ++j) {
     if (K[j]) {
       atomicAdd(d.k + c[j], K[j]);
       atomicAdd(d.a + c[j], A[j]);
@@ -672,16 +673,16 @@ struct MomSums {
 };
 // e with x < 2^e for 0 <= x < bound
 __device__ __forceinline__ int mom_bound(float bound) { return bound > 0.0f ? max(ilogbf(bound) + 1, -100) : -100; }
-// one quantity (0: J.E, 1, 2: first moments, 3, 4: second) of four particles,
+// one quantity (0: J.E, 1, 2: first moments, 3, 4: second) of V particles,
 // runs of equal cells merged (c[j] < 0: none)
-template <int Q>
-__device__ __forceinline__ void mom_add4(const MomSums& m, const int c[4], const float x[4]) {
+template <int Q, int V>
+__device__ __forceinline__ void mom_add4(const MomSums& m, const int c[V], const float x[V]) {
   constexpr int kind = (Q + 1) / 2;
   double* far = Q == 0 ? m.pw : m.md + (Q >= 3 ? m.N + 1 : 0) + ((Q & 1) ? 0 : 1);
-  int hi[4];
-  unsigned mid[4], lo[4];
+  int hi[V];
+  unsigned mid[V], lo[V];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < V; ++j) {
     const unsigned u = __float_as_uint(x[j]);
     const int sh = (int)((u >> 23) & 0xFFu) - 127 - m.e[kind] + 24;
     const bool in = c[j] >= 0 && sh >= 0 && sh < 24 && (unsigned)(c[j] - m.w0) < (unsigned)m.w;
@@ -693,7 +694,7 @@ __device__ __forceinline__ void mom_add4(const MomSums& m, const int c[4], const
     hi[j] = (int)(t >> 32);
   }
 #pragma unroll
-  for (int j = 3; j >= 1; --j)
+  for (int j = V - 1; j >= 1; --j)
     if (c[j] >= 0 && c[j] == c[j - 1]) {
       hi[j - 1] += hi[j];
       mid[j - 1] += mid[j];
@@ -703,7 +704,7 @@ __device__ __forceinline__ void mom_add4(const MomSums& m, const int c[4], const
     }
   int* base = m.words + (3 * Q) * m.w - m.w0;
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+  for (int j = 0; j < V; ++j)
     if (hi[j] | (int)(mid[j] | lo[j])) {
       atomicAdd(base + c[j], hi[j]);
       atomicAdd(base + m.w + c[j], (int)mid[j]);
@@ -731,11 +732,12 @@ __device__ __forceinline__ void mom_flush(const MomSums& m) {
 
 // The key of a lane's valid entries c[j] >= 0: their common cell, -1 if they
 // lie in several cells or there are none.
-__device__ __forceinline__ int lane_cell_key(const int c[4]) {
+template <int V>
+__device__ __forceinline__ int lane_cell_key(const int (&c)[V]) {
   int k = -1;
   bool multi = false;
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+  for (int j = 0; j < V; ++j)
     if (c[j] >= 0) {
       if (k < 0) k = c[j];
       else if (c[j] != k) multi = true;
@@ -772,11 +774,13 @@ __device__ __forceinline__ void l2_prefetch(const void* p, unsigned bytes) {
 // FUSED (k_steps): the real collisions are carried out where they are found,
 // and impacts tallied, instead of being recorded for k_collide; a block of
 // BLOCK threads with twice the registers of k_pass's.
-template <int KIND, bool STAGE, int BLOCK, bool FUSED>
+template <int KIND, bool STAGE, int BLOCK, bool FUSED, int V = 4>
 __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, const SegDev& G, int s,
                            const PieceState& ps, long long qbeg, long long qend, int mode, uint32_t* dep,
                            float* Msm, unsigned char* ring, PassShared& sh, FusedStep* fx = nullptr,
                            const float* field = nullptr, int mom_words = 0) {
+  // (indices of the four-particle vector loads, which only V = 4 reaches)
+  constexpr int x1 = V > 1 ? 1 : 0, x2 = V > 2 ? 2 : 0, x3 = V > 3 ? 3 : 0;
   const int slot = G.run, sp = G.species;
   RunState* st = b.rst + slot;
   SegState* ss = b.sst + s;
@@ -841,11 +845,11 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
     for (int i = threadIdx.x; i < ne; i += BLOCK) em = fmaxf(em, fabsf(E[i]));
     for (long long q = qbeg + threadIdx.x; q < qend; q += BLOCK) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float a = 4 * q + j < n ? fabsf(pvx[4 * q + j]) : 0.0f;
+      for (int j = 0; j < V; ++j) {
+        const float a = V * q + j < n ? fabsf(pvx[V * q + j]) : 0.0f;
         vm = a < 3.0e8f ? fmaxf(vm, a) : vm;  // (the others fail the run)
       }
-      if (mom.w < N && pc[4 * q] >= 0) lowest = min(lowest, pc[4 * q]);
+      if (mom.w < N && pc[V * q] >= 0) lowest = min(lowest, pc[V * q]);
     }
     const unsigned eb = __reduce_max_sync(kFull, __float_as_uint(em));
     const unsigned vb = __reduce_max_sync(kFull, __float_as_uint(vm));
@@ -901,7 +905,7 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
   for (long long base = qbeg;; base += BLOCK) {
     const bool more = base < qend;
     if (more) {
-      if (threadIdx.x == 0) {
+      if (V == 4 && threadIdx.x == 0) {
         // the next iteration's particle records into L2
         const long long nb = base + BLOCK;
         if (nb < qend) {
@@ -925,21 +929,21 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         }
       }
       const long long q = base + (long long)threadIdx.x;
-      const long long i0 = 4 * q;
+      const long long i0 = V * q;
       const bool inq = q < qend && chk(i0 < G.cap, 2, i0, G.cap);
-      const bool full = inq && (i0 + 3 < n) && chk(i0 + 3 < G.cap, 3, i0 + 3, G.cap);
-      int c[4];
-      float f[4], v[4];
+      const bool full = V == 4 && inq && (i0 + 3 < n) && chk(i0 + 3 < G.cap, 3, i0 + 3, G.cap);
+      int c[V];
+      float f[V], v[V];
       if (full) {
         const int4 c4 = *reinterpret_cast<const int4*>(pc + i0);
         const float4 f4 = *reinterpret_cast<const float4*>(pxi + i0);
         const float4 v4 = *reinterpret_cast<const float4*>(pvx + i0);
-        c[0] = c4.x; c[1] = c4.y; c[2] = c4.z; c[3] = c4.w;
-        f[0] = f4.x; f[1] = f4.y; f[2] = f4.z; f[3] = f4.w;
-        v[0] = v4.x; v[1] = v4.y; v[2] = v4.z; v[3] = v4.w;
+        c[0] = c4.x; c[x1] = c4.y; c[x2] = c4.z; c[x3] = c4.w;
+        f[0] = f4.x; f[x1] = f4.y; f[x2] = f4.z; f[x3] = f4.w;
+        v[0] = v4.x; v[x1] = v4.y; v[x2] = v4.z; v[x3] = v4.w;
       } else {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < V; ++j) {
           const bool in = inq && (i0 + j < n);
           c[j] = in ? pc[i0 + j] : -1;
           f[j] = in ? pxi[i0 + j] : 0.0f;
@@ -948,61 +952,66 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
       }
       // weight multipliers: read here on sample steps (the moments use them),
       // else just before the deposit (a shorter live range)
-      unsigned kq[4] = {1u, 1u, 1u, 1u};
+      unsigned kq[V];
+#pragma unroll
+      for (int j = 0; j < V; ++j) kq[j] = 1u;
       if (weighted && sample) {
         if (full) {
           const uint4 k4 = *reinterpret_cast<const uint4*>(pwt + i0);
-          kq[0] = k4.x; kq[1] = k4.y; kq[2] = k4.z; kq[3] = k4.w;
+          kq[0] = k4.x; kq[x1] = k4.y; kq[x2] = k4.z; kq[x3] = k4.w;
         } else {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) kq[j] = (inq && i0 + j < n) ? pwt[i0 + j] : 1u;
+          for (int j = 0; j < V; ++j) kq[j] = (inq && i0 + j < n) ? pwt[i0 + j] : 1u;
         }
       }
-      bool cand[4] = {false, false, false, false};
+      bool cand[V] = {};
       unsigned hit = 0u;  // bit j: absorbed at x = 0 (impact tallies)
-      if ((c[0] | c[1] | c[2] | c[3]) >= 0) {
-        nlive += 4u;
+      int any = c[0];  // negative: some particle is absorbed
+#pragma unroll
+      for (int j = 1; j < V; ++j) any |= c[j];
+      if (any >= 0) {
+        nlive += (unsigned)V;
       } else {
         // absorbed particles: far from every cell, wherever the push takes them
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < V; ++j) {
           nlive += c[j] >= 0 ? 1u : 0u;
           c[j] = c[j] >= 0 ? c[j] : kFarCell;
         }
       }
       if (stepping) {
-        uint64_t id[4] = {0, 0, 0, 0};
+        uint64_t id[V] = {};
         if (mcc) {
           if (full) {
             const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(pid + i0);
             const ulonglong2 bq = *reinterpret_cast<const ulonglong2*>(pid + i0 + 2);
-            id[0] = a.x; id[1] = a.y; id[2] = bq.x; id[3] = bq.y;
+            id[0] = a.x; id[x1] = a.y; id[x2] = bq.x; id[x3] = bq.y;
           } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) id[j] = c[j] >= 0 ? pid[i0 + j] : 0ull;
+            for (int j = 0; j < V; ++j) id[j] = c[j] >= 0 ? pid[i0 + j] : 0ull;
           }
         }
         // vy^2 + vz^2 (collisions do not change it before the push reads it)
-        float yz[4] = {0.f, 0.f, 0.f, 0.f};
+        float yz[V] = {};
         if (load_yz) {
           if (full) {
             const float4 y4 = *reinterpret_cast<const float4*>(pvy + i0);
             const float4 z4 = *reinterpret_cast<const float4*>(pvz + i0);
             yz[0] = yz2(y4.x, z4.x);
-            yz[1] = yz2(y4.y, z4.y);
-            yz[2] = yz2(y4.z, z4.z);
-            yz[3] = yz2(y4.w, z4.w);
+            yz[x1] = yz2(y4.y, z4.y);
+            yz[x2] = yz2(y4.z, z4.z);
+            yz[x3] = yz2(y4.w, z4.w);
           } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
+            for (int j = 0; j < V; ++j)
               if (c[j] >= 0) yz[j] = yz2(pvy[i0 + j], pvz[i0 + j]);
           }
         }
         // gather (Eq. 6-7; CIC for MC) and push (Eq. 8), branch-free over the
         // four particles so the loads and arithmetic overlap
-        float Ei[4];
+        float Ei[V];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < V; ++j) {
           if (!chk(c[j] < N, 4, c[j], N)) c[j] = kFarCell;
           const int cc = max(c[j], 0);
           if (scheme == ECPIC_SCHEME_EC) {
@@ -1038,9 +1047,9 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         }
         float keq = 0.0f;
         Float2 kef{0.0f, 0.0f};  // k_steps: the quad's terms without rounding their sum
-        float pje[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        float pje[V] = {};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < V; ++j) {
           const float vnew = v[j] + qm_dt * Ei[j];
           if (sample) {
             const float fk = weighted ? (float)kq[j] : 1.0f;
@@ -1059,11 +1068,11 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
           const int key = lane_cell_key(c);
           double* pwg = R->pw + (size_t)sp * N;
           if (fixed) {
-            mom_add4<0>(mom, c, pje);
+            mom_add4<0, V>(mom, c, pje);
           } else if (FUSED) {
             Float2 pl{0.0f, 0.0f};
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < V; ++j) {
               if (c[j] < 0) continue;
               if (key < 0) atomicAdd(pwg + c[j], (double)pje[j]);
               else pl.add(pje[j]);
@@ -1076,7 +1085,7 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
           float pl = 0.0f;
           int cc = -1;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < V; ++j) {
             if (c[j] < 0) continue;
             if (key < 0 && c[j] != cc) {
               if (cc >= 0) atomicAdd(pwg + cc, (double)pl);
@@ -1097,10 +1106,10 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         }
         // Philox block A of all four: independent chains the scheduler
         // interleaves; A.x decides the candidate, A.y selects the process
-        uint32_t r0[4] = {0u, 0u, 0u, 0u}, ry[4] = {0u, 0u, 0u, 0u};
+        uint32_t r0[V] = {}, ry[V] = {};
         if (mcc) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < V; ++j) {
             const uint4 A = draw(seed, id[j], (uint32_t)k, (uint32_t)sp << 8);
             r0[j] = A.x;
             ry[j] = A.y;
@@ -1108,12 +1117,12 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         }
         // Eq. 9 in cell units, then the walls: absorbed when X <= 0 or X >= L
 #pragma unroll
-        for (int j = 0; j < 4; ++j) cand[j] = mcc && r0[j] <= thr_last;
+        for (int j = 0; j < V; ++j) cand[j] = mcc && r0[j] <= thr_last;
         if (uniform) {
-          int cj[4];
-          float g[4];
+          int cj[V];
+          float g[V];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < V; ++j) {
             g[j] = f[j] + v[j] * dtdx_u;
             const float fl = floorf(g[j]);
             cj[j] = c[j] + (int)fl;
@@ -1123,20 +1132,24 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
           // X = 0, offsets that did not round to 1 and finite speeds.  One set
           // of tests per quad sees that (some tests wider than the rule); the
           // others are told apart particle by particle in a rare branch.
-          const unsigned top = max(max((unsigned)cj[0], (unsigned)cj[1]), max((unsigned)cj[2], (unsigned)cj[3]));
-          const unsigned zero = min(min((unsigned)cj[0] | __float_as_uint(g[0]), (unsigned)cj[1] | __float_as_uint(g[1])),
-                                    min((unsigned)cj[2] | __float_as_uint(g[2]), (unsigned)cj[3] | __float_as_uint(g[3])));
-          const float gm = fmaxf(fmaxf(g[0], g[1]), fmaxf(g[2], g[3]));
-          const float vs = (fabsf(v[0]) + fabsf(v[1])) + (fabsf(v[2]) + fabsf(v[3]));
+          unsigned top = 0u, zero = 0xFFFFFFFFu;
+          float gm = 0.0f, vs = 0.0f;
+#pragma unroll
+          for (int j = 0; j < V; ++j) {
+            top = max(top, (unsigned)cj[j]);
+            zero = min(zero, (unsigned)cj[j] | __float_as_uint(g[j]));
+            gm = fmaxf(gm, g[j]);
+            vs += fabsf(v[j]);
+          }
           if (top < (unsigned)N && zero != 0u && gm < 1.0f && vs < 3.0e8f) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < V; ++j) {
               c[j] = cj[j];
               f[j] = g[j];
             }
           } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < V; ++j) {
               bool ok = c[j] >= 0;
               if (ok) {
                 if (g[j] >= 1.0f) {  // g - floor(g) rounded to 1
@@ -1167,7 +1180,7 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
           }
         } else {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < V; ++j) {
             if (c[j] < 0) {
               c[j] = -1;
               cand[j] = false;
@@ -1195,12 +1208,12 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
           }
         }
         if (full) {
-          *reinterpret_cast<int4*>(pc + i0) = make_int4(c[0], c[1], c[2], c[3]);
-          *reinterpret_cast<float4*>(pxi + i0) = make_float4(f[0], f[1], f[2], f[3]);
-          *reinterpret_cast<float4*>(pvx + i0) = make_float4(v[0], v[1], v[2], v[3]);
+          *reinterpret_cast<int4*>(pc + i0) = make_int4(c[0], c[x1], c[x2], c[x3]);
+          *reinterpret_cast<float4*>(pxi + i0) = make_float4(f[0], f[x1], f[x2], f[x3]);
+          *reinterpret_cast<float4*>(pvx + i0) = make_float4(v[0], v[x1], v[x2], v[x3]);
         } else {
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
+          for (int j = 0; j < V; ++j)
             if (inq && i0 + j < n) {
               pc[i0 + j] = c[j];
               pxi[i0 + j] = f[j];
@@ -1211,7 +1224,7 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         // collision kernel (the absorbed slot keeps its velocity until the sort)
         if (imp_on && __any_sync(kFull, hit != 0u)) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < V; ++j) {
             const unsigned m = __ballot_sync(kFull, (hit >> j) & 1u);
             if (m) {
               const int lead = __ffs(m) - 1;
@@ -1232,7 +1245,7 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         // collision kernel moves the particles that collide)
         if (eedf_on) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
+          for (int j = 0; j < V; ++j)
             if (c[j] >= ec0 && c[j] <= ec1)
               atomicAdd(tal + tally_bin(kin_eV(SP->half_m_over_e, v[j], yz[j]), R->eedf_dEinv, R->eedf_n),
                         (unsigned long long)kq[j]);
@@ -1245,7 +1258,7 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
           // rounded up: the test itself decides what this lets through.
           unsigned mine = 0u;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < V; ++j) {
             ncand += cand[j] ? 1u : 0u;
             const float Rl = (__uint_as_float((ry[j] >> 9) | 0x3F800000u) - 1.0f) * nu_max;
             const bool null = yz_stream && Rl * Rl > nu_bnd2 * (v[j] * v[j] + yz[j]);
@@ -1268,51 +1281,51 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
       // fixed-point CIC deposit of the new positions (Eq. 2-3); vx moments
       // (pre-collision: the collision adds the change)
       if (order2)
-        dep2_add4(dlo, dhi, N, !walls, c, f);
+        dep2_add4<V>(dlo, dhi, N, !walls, c, f);
       else if (weighted) {
         if (!sample) {
           if (full) {
             const uint4 k4 = *reinterpret_cast<const uint4*>(pwt + i0);
-            kq[0] = k4.x; kq[1] = k4.y; kq[2] = k4.z; kq[3] = k4.w;
+            kq[0] = k4.x; kq[x1] = k4.y; kq[x2] = k4.z; kq[x3] = k4.w;
           } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) kq[j] = (inq && i0 + j < n) ? pwt[i0 + j] : 1u;
+            for (int j = 0; j < V; ++j) kq[j] = (inq && i0 + j < n) ? pwt[i0 + j] : 1u;
           }
         }
-        depw_add4(dw, c, f, kq);
+        depw_add4<V>(dw, c, f, kq);
       }
       else
-        dep_add4(dcnt, dlo, dhi, c, f);
+        dep_add4<V>(dcnt, dlo, dhi, c, f);
       if (sample) {
         // vx moments at the nodes of the new cell (CIC shares): per lane
         // summed where its particles share a cell, then down each segment
         const int Nm = b.nmax + 1;
-        int cm[4];
+        int cm[V];
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < V; ++j)
           cm[j] = (c[j] >= 0 && chk(c[j] + 1 <= b.nmax, 20, c[j], b.nmax)) ? c[j] : -1;
         const int key = lane_cell_key(cm);
         double* mdg = R->momd + (size_t)sp * 2 * (N + 1);
         if (fixed) {
-          float x[4], y[4];
+          float x[V], y[V];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < V; ++j) {
             x[j] = (1.0f - f[j]) * v[j];
             y[j] = x[j] * v[j];
           }
-          mom_add4<1>(mom, cm, x);
-          mom_add4<3>(mom, cm, y);
+          mom_add4<1, V>(mom, cm, x);
+          mom_add4<3, V>(mom, cm, y);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < V; ++j) {
             x[j] = f[j] * v[j];
             y[j] = x[j] * v[j];
           }
-          mom_add4<2>(mom, cm, x);
-          mom_add4<4>(mom, cm, y);
+          mom_add4<2, V>(mom, cm, x);
+          mom_add4<4, V>(mom, cm, y);
         } else if (FUSED) {
           Float2 a1{0.0f, 0.0f}, b1{0.0f, 0.0f}, a2{0.0f, 0.0f}, b2{0.0f, 0.0f};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < V; ++j) {
             if (cm[j] < 0) continue;
             const float fk = weighted ? (float)kq[j] : 1.0f;
             const float lo = fk * ((1.0f - f[j]) * v[j]), hi = fk * (f[j] * v[j]);
@@ -1345,7 +1358,7 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
         float a1 = 0.0f, b1 = 0.0f, a2 = 0.0f, b2 = 0.0f;
         int cc = -1;  // spread lanes: the current run of equal cells
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < V; ++j) {
           if (cm[j] < 0) continue;
           const float fk = weighted ? (float)kq[j] : 1.0f;
           const float lo = fk * ((1.0f - f[j]) * v[j]), hi = fk * (f[j] * v[j]);
@@ -1476,7 +1489,7 @@ __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, 
       }
     }
     if (!more) break;
-    constexpr int iters = kFlushParticles / (4 * BLOCK);
+    constexpr int iters = kFlushParticles / (V * BLOCK);
     if (++since_flush == (order2 ? iters / 4 : weighted ? iters / 2 : iters)) {
       __syncthreads();
       if (order2)
