@@ -295,6 +295,7 @@ int ecpic_init(ecpic_run* r, uint64_t seed, double dt, const int64_t* n_per_spec
     r->spec.T_eV.assign(T_eV, T_eV + ns);
     const std::string v = ecpic::validate_spec(r->spec);
     if (!v.empty()) return fail(r, ECPIC_ERR_ARG, v);
+    ecpic::set_null_rates(&r->spec);
     const int N = (int)r->spec.edges.size() - 1;
     std::unique_ptr<Batch> b(new Batch(r->device, r->stream, 1, (int)ns, N));
     b->set_sort_every(r->sort_every);

@@ -127,6 +127,7 @@ int spec_from_config(const ecpic_run_config* c, int64_t n_steps, RunSpec* s, std
     *err = v;
     return ECPIC_ERR_ARG;
   }
+  ecpic::set_null_rates(s);
   return ECPIC_OK;
 }
 

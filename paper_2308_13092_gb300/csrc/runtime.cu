@@ -49,9 +49,9 @@ struct Carve {
 // null-collision probability P; mean + 12 standard deviations + 256 is never
 // exceeded in practice (an overflow fails the run with ECPIC_ERR_CAPACITY).
 long long real_capacity(const HostSpecies& sp, const RunSpec& s) {
-  double nu = 0.0;
-  uint32_t thr = 0;
-  null_rate(sp, s, &nu, &thr);
+  double nu = sp.nu;
+  uint32_t thr = sp.thr24;
+  if (!sp.rated) null_rate(sp, s, &nu, &thr);
   if (thr == 0 || sp.cap <= 0) return 0;
   const double mean = (double)sp.cap * ((double)thr / 16777216.0);
   const double bound = std::ceil(mean + 12.0 * std::sqrt(mean) + 256.0);
@@ -293,6 +293,13 @@ void null_rate(const HostSpecies& sp, const RunSpec& s, double* nu_max, uint32_t
   double t = std::ceil(P * 16777216.0);
   if (t > 16777216.0) t = 16777216.0;
   *thr24 = (uint32_t)t;
+}
+
+void set_null_rates(RunSpec* s) {
+  for (HostSpecies& sp : s->species) {
+    null_rate(sp, *s, &sp.nu, &sp.thr24);
+    sp.rated = true;
+  }
 }
 
 size_t run_bytes(const RunSpec& s) { return layout_bytes(s); }
@@ -641,9 +648,9 @@ int Batch::admit(int slot, const RunSpec& spec, std::string* err, bool defer) {
     D.two_m_over_M = (float)(2.0 * hs.m / mg);
     D.m_frac = (float)(mg / (hs.m + mg));
     D.mass_frac = (float)(hs.m / (hs.m + mg));
-    double nu;
-    uint32_t thr;
-    null_rate(hs, spec, &nu, &thr);
+    double nu = hs.nu;
+    uint32_t thr = hs.thr24;
+    if (!hs.rated) null_rate(hs, spec, &nu, &thr);
     D.nu_max = (float)nu;
     D.thr24 = thr;
     D.nproc = (int)hs.procs.size();

@@ -22,6 +22,12 @@ struct HostSpecies {
   double q = 0, m = 0, w = 0;
   long long cap = 0;
   std::vector<HostProc> procs;
+  // null-collision bound and threshold, once set_null_rates has formed them:
+  // they run over the whole cross-section table (a square root and a division
+  // per entry, about 20 us for 2000), and a run's sizes ask for them four times
+  bool rated = false;
+  double nu = 0;
+  uint32_t thr24 = 0;
 };
 
 struct RunSpec {
@@ -62,6 +68,7 @@ std::string validate_tallies(const RunSpec& s);
 // null-collision bound of a species (FP64, host): nu_max and the 24-bit
 // candidate threshold
 void null_rate(const HostSpecies& sp, const RunSpec& s, double* nu_max, uint32_t* thr24);
+void set_null_rates(RunSpec* s);  // of a complete run description
 // bytes of device memory a run needs
 size_t run_bytes(const RunSpec& s);
 
