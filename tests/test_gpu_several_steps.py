@@ -32,8 +32,8 @@ def _tanh(scheme, n=5003):
     return _ccp(0, n, 5, scheme=scheme, edges=I.tanh_edges(101, 0.05, 1e-4))
 
 
-def _rebalanced(scheme):
-    c = _tanh(scheme, 9001)
+def _rebalanced(scheme, n=9001):
+    c = _tanh(scheme, n)
     c.rebalance = dict(every=5, target=64, lo=40, hi=80, m0=16)
     return c
 
@@ -61,6 +61,11 @@ CASES = {
     "periodic mc2": lambda: I.periodic_plasma(N=65, ppc=33, scheme=I.MC2, ions=False, seed=4),
     "rebalanced ec": lambda: _rebalanced(I.EC),
     "rebalanced mc": lambda: _rebalanced(I.MC),
+    # two particles per thread
+    "ec, 60000": lambda: _ccp(128, 30001, 10),
+    "ec2, 60000": lambda: _ccp(97, 30002, 11, scheme=I.EC2),
+    "rebalanced ec, 60000": lambda: _rebalanced(I.EC, 30003),
+    "rebalanced mc, 60000": lambda: _rebalanced(I.MC, 30003),
 }
 
 
