@@ -34,6 +34,7 @@ constexpr int kOnlyFresh = -2;
 struct InitParams {
   long long n[kMaxSpecies];
   double sd[kMaxSpecies];  // sqrt(e T / m)
+  float sd_hi[kMaxSpecies], sd_lo[kMaxSpecies];  // the same as two floats
   int quiet;               // positions X_i = (i + 1/2) L / n instead of Philox
   unsigned rb_m0;          // weight multiplier of loaded particles (rebalancing runs)
 };

@@ -748,6 +748,8 @@ int Batch::admit(int slot, const RunSpec& spec, std::string* err, bool defer) {
   for (int s = 0; s < ns; ++s) {
     ip.n[s] = spec.n_init[s];
     ip.sd[s] = std::sqrt(kQe * spec.T_eV[s] / spec.species[s].m);
+    ip.sd_hi[s] = (float)ip.sd[s];
+    ip.sd_lo[s] = (float)(ip.sd[s] - (double)ip.sd_hi[s]);
   }
   if (defer) {
     wave_slots_.push_back(slot);
