@@ -215,7 +215,8 @@ int ecpic_set_tallies(ecpic_run* run, double eedf_center_m, double eedf_halfwidt
  * solve the field of step 0.  Allocates all device memory. */
 int ecpic_init(ecpic_run* run, uint64_t seed, double dt_s,
                const int64_t* n_per_species, const double* T_eV);
-/* Advance n_steps (async).  One step: EC (or MC) gather and leapfrog push
+/* Advance n_steps (async; a run or batch that does not fill the device takes
+ * several steps per launch, others replay a graph of launches).  One step: EC (or MC) gather and leapfrog push
  * (Eq. 6-9), wall absorption, null-collision MCC, CIC deposit (Eq. 2-3),
  * Poisson (Eq. 4) and field (Eq. 5) of the next time level. */
 int ecpic_step(ecpic_run* run, int64_t n_steps);
@@ -263,7 +264,8 @@ int ecpic_set_auto_grow(ecpic_run* run, int on);
  * counting sort and the real-collision kernel; launches[0..3] = their launch
  * counts.  Same physics as ecpic_step. */
 int ecpic_profile_step(ecpic_run* run, int64_t n_steps, double* ms, int64_t* launches);
-/* Pass-kernel grid size override (0 = automatic); for tuning. */
+/* Pass-kernel grid size override (0 = automatic); for tuning.  A run with an
+ * override takes a launch per kernel phase. */
 int ecpic_set_pass_grid(ecpic_run* run, int ctas);
 /* Autotuner over the sort cadence K and the particles per CTA: times the
  * graph-replayed step for each candidate pair of counting-sort cadence K in
@@ -290,7 +292,8 @@ int ecpic_autotune_ks(ecpic_run* run, int64_t steps_per_trial, const int* ks, in
  * step that ecpic_step advances from then on adds the device time of its
  * phases (CUDA events on the run's stream) to running sums.  The sums thus
  * come from the very replays that advance the run, not from a separate
- * profiling pass.  on = 0 restores the plain graphs (the sums are kept). */
+ * profiling pass.  While it is on, a run that would take several steps per
+ * launch takes a launch per phase instead, with the same results.  on = 0 restores the plain graphs (the sums are kept). */
 int ecpic_set_phase_timing(ecpic_run* run, int on);
 /* Read and clear the phase sums (waits for the timed steps): ms[0..3] = the
  * particle pass, the field solve, the counting sort, the real-collision

@@ -1,11 +1,13 @@
 // kernels.cu -- the sm_103a kernels of libecpic.
 //
-// One time step of every resident run is two launches:
+// One time step of every resident run is three launches (batches bound by
+// latency take several steps per launch instead: steps.cuh):
 //   k_pass   fused gather (Eq. 6-7, or CIC for the MC scheme) -> leapfrog
 //            push (Eq. 8-9) in cell-relative FP32 -> wall absorption ->
 //            null-collision MCC (Sec. 2a step 6) -> fixed-point CIC deposit
 //            (Eq. 2-3) of the new positions, over all (run, species)
 //            segments, load-balanced by particle count;
+//   k_collide the real collisions and impacts that the pass recorded;
 //   k_field  per run: charge from the deposit, Poisson (Eq. 4) in its
 //            two-scan form, field (Eq. 5 or centred), potential, sampling.
 // Every K steps a counting sort by cell (k_hist, k_scan, k_scatter,

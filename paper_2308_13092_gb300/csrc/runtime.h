@@ -1,6 +1,7 @@
 // runtime.h -- host runtime of libecpic: a Batch owns the device state of up
-// to max_slots independent runs and steps them together (one launch per
-// phase for all runs, replayed from CUDA graphs).
+// to max_slots independent runs and steps them together: one launch per
+// phase for all runs, replayed from CUDA graphs, or, where the batch is bound by
+// latency (several_steps), several steps per cooperative launch.
 #pragma once
 #include <climits>
 #include <cstdint>

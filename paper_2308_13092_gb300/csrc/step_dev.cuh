@@ -752,11 +752,13 @@ __device__ __forceinline__ void l2_prefetch(const void* p, unsigned bytes) {
 }
 
 // Streaming part of one piece: quads [qbeg, qend) of segment s, four
-// particles per thread with 16-byte loads.  Gather (Eq. 6-7 / CIC), leapfrog
+// particles per thread with 16-byte loads (V: or two, or one, where a block of
+// k_steps has few).  Gather (Eq. 6-7 / CIC), leapfrog
 // (Eq. 8-9) in cell units, walls, the Philox candidate test, fixed-point
 // deposit of X^{k+1} (Eq. 2-3).  Collision candidates (Sec. 2a step 6)
-// enter a per-warp ring with their selection word and |g|^2 (or vx); the
-// warp drains it 32 at a time (all lanes busy) with the null-collision test.
+// enter a per-warp ring by their index; the warp drains it 32 at a time (all
+// lanes busy): it reads the pushed particle again, redraws its Philox block and
+// makes the null-collision test.
 // The few real collisions are recorded for k_collide, which scatters them
 // with its own register budget.  vy, vz are streamed when a species'
 // candidate probability is 1/16 or more (its candidates then touch most
@@ -773,7 +775,7 @@ __device__ __forceinline__ void l2_prefetch(const void* p, unsigned bytes) {
 //
 // FUSED (k_steps): the real collisions are carried out where they are found,
 // and impacts tallied, instead of being recorded for k_collide; a block of
-// BLOCK threads with twice the registers of k_pass's.
+// 512 or 256 threads with two or four times the registers of k_pass's.
 template <int KIND, bool STAGE, int BLOCK, bool FUSED, int V = 4>
 __device__ __forceinline__ void pass_piece(const BatchView& b, const RunDev* R, const SegDev& G, int s,
                            const PieceState& ps, long long qbeg, long long qend, int mode, uint32_t* dep,
