@@ -1333,6 +1333,13 @@ bool Batch::several_steps() {
 }
 
 int Batch::step_several(long long n, std::string* err) {
+  // refused under a caller's capture, as the step graphs are: the levels and
+  // sort cycles counted here would part from what the graph replays
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  int rc0 = check(cudaStreamIsCapturing(stream_, &cap), "step", err);
+  if (rc0 == ECPIC_OK && cap != cudaStreamCaptureStatusNone)
+    rc0 = check(cudaErrorStreamCaptureUnsupported, "step", err);
+  if (rc0) return rc0;
   const BatchView b = view();
   while (n > 0) {
     const int m = rb_first_due((int)std::min<long long>(n, kStepsPerLaunch));

@@ -123,3 +123,24 @@ def test_batch_of_different_runs():
         assert d["step"] == e["step"] == n and d["species"] == e["species"]
         assert np.array_equal(d["density"], e["density"])
         assert np.allclose(d["phi"], e["phi"], rtol=0, atol=1e-12 * max(1.0, np.abs(e["phi"]).max()))
+
+
+def test_step_under_capture_is_refused():
+    """A step counts levels on the host, so a caller's graph cannot hold it:
+    the error leaves the run as it was."""
+    import torch
+    from paper_2308_13092_gb300 import ecpic
+    s = torch.cuda.Stream()
+    r, a = (ecpic.Run.from_config(CASES["ec"](), stream=s.cuda_stream) for _ in range(2))
+    for x in (r, a):
+        x.step(20)
+        x.sync()
+    with pytest.raises(Exception):
+        with torch.cuda.graph(torch.cuda.CUDAGraph(), stream=s):
+            r.step(1)
+    for x in (r, a):
+        x.step(20)
+        x.sync()
+    assert r.diagnostics()["step"] == 40
+    for u, v in zip(_state(r)[2], _state(a)[2]):
+        assert all(np.array_equal(x, y) for x, y in zip(u, v))
