@@ -8,7 +8,7 @@ bool steps_fit(const BatchView& b, int device) {
   int most = 0, coop = 0;
   cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device);
-  return coop != 0 && steps_smem(b, 512) + 1024 <= (size_t)most;
+  return coop != 0 && kStepSmem + 1024 <= (size_t)most && steps_smem(b, 512) <= kStepSmem;
 }
 
 cudaError_t launch_steps(const BatchView& b, const StepPlan& pl, const StepTeams& tm, int steps, int sort_every,

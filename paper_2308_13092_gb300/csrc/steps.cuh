@@ -824,6 +824,7 @@ __global__ void __launch_bounds__(kStepBlock, 1)
   flush_counters<kStepBlock>(sh, st, sst, ns);
 }
 
+constexpr size_t kStepSmem = 226 * 1024;  // dynamic shared memory of a block, at most
 size_t steps_smem(const BatchView& b, int threads) {
   return steps_bytes(b.nmax, b.nseg / b.max_slots, b.weighted != 0, threads);
 }
@@ -832,7 +833,9 @@ template <bool W, int kStepBlock, int V>
 cudaError_t launch_w(const BatchView& b, const StepPlan& pl, const StepTeams& tm, int steps, int sort_every,
                      int since_sort, cudaStream_t s) {
   const size_t sm = steps_smem(b, kStepBlock);
-  cudaError_t e = cudaFuncSetAttribute(k_steps<W, kStepBlock, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  // the same limit on every call: threads with runs of other sizes set it too
+  cudaError_t e = cudaFuncSetAttribute(k_steps<W, kStepBlock, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kStepSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)tm.blocks);

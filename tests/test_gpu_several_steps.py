@@ -125,6 +125,33 @@ def test_batch_of_different_runs():
         assert np.allclose(d["phi"], e["phi"], rtol=0, atol=1e-12 * max(1.0, np.abs(e["phi"]).max()))
 
 
+def test_runs_in_several_threads():
+    """Runs of different sizes stepped from several threads, each on its own
+    stream, against the same runs alone."""
+    import threading
+    cfgs = [_ccp(64 + 400 * k, 3000 * (k + 1), 20 + k) for k in range(5)]
+
+    def advance(c, out, k):
+        r = gpu_from_config(c)
+        for _ in range(40):
+            r.step(5)
+        r.sync()
+        out[k] = _state(r)[2]
+
+    alone, at_once = [None] * 5, [None] * 5
+    for k, c in enumerate(cfgs):
+        advance(c, alone, k)
+    t = [threading.Thread(target=advance, args=(c, at_once, k)) for k, c in enumerate(cfgs)]
+    for x in t:
+        x.start()
+    for x in t:
+        x.join()
+    for a, b in zip(alone, at_once):
+        assert b is not None
+        for u, v in zip(a, b):
+            assert all(np.array_equal(x, y) for x, y in zip(u, v))
+
+
 def test_step_under_capture_is_refused():
     """A step counts levels on the host, so a caller's graph cannot hold it:
     the error leaves the run as it was."""
