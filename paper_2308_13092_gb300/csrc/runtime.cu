@@ -404,9 +404,16 @@ Batch::Batch(int device, cudaStream_t stream, int max_slots, int spc, int nmax)
   cudaMalloc(&d_rblist_, sizeof(int) * (size_t)nseg_ * nmax_);
   cudaMalloc(&d_rbnum_, sizeof(int));
   if (max_slots_ <= std::min(sm_count_, kMaxStepBlocks)) {
-    cudaMalloc(&plan_.words, sizeof(StepWords) * (size_t)max_slots_);
-    cudaMalloc(&plan_.deposit, plan_deposit_bytes() * (size_t)max_slots_);
-    cudaMemsetAsync(plan_.deposit, 0, plan_deposit_bytes() * (size_t)max_slots_, stream_);
+    // without room for it the batch takes a launch per phase
+    if (cudaMalloc(&plan_.words, sizeof(StepWords) * (size_t)max_slots_) != cudaSuccess ||
+        cudaMalloc(&plan_.deposit, plan_deposit_bytes() * (size_t)max_slots_) != cudaSuccess) {
+      cudaGetLastError();
+      cudaFree(plan_.words);
+      plan_.words = nullptr;
+      plan_.deposit = nullptr;
+    } else {
+      cudaMemsetAsync(plan_.deposit, 0, plan_deposit_bytes() * (size_t)max_slots_, stream_);
+    }
   }
   cudaMalloc(&d_wave_slots_, sizeof(int) * max_slots_);
   cudaMalloc(&d_wave_params_, sizeof(InitParams) * max_slots_);
