@@ -660,9 +660,12 @@ __device__ __forceinline__ Float2 warp_seg_sum(Float2 x, unsigned heads) {
 // float term x of at least 2^(e-24) is the 48-bit integer x 2^(47-e) exactly;
 // its signed high and unsigned lower 16-bit parts go to the words.  Smaller
 // terms, and cells outside the window that the shared memory holds, are
-// added straight to the run's FP64 sums in HBM.  So the sums are exact and the
-// same in any order.  At most kFlushParticles particles between flushes keep
-// every word in range.
+// added straight to the run's FP64 sums in HBM.  So the sums of the terms are
+// exact and the same in any order; the terms, the second moments' products
+// included, are the floats that k_pass forms for a particle by itself (products
+// without that rounding leave the sums farther from k_pass's: 1.2e-8 against
+// 4e-9 with 6 particles per cell).  At most kFlushParticles particles between
+// flushes keep every word in range.
 constexpr int kMomSums = 5;
 struct MomSums {
   int* words;          // [quantity][part][w]
