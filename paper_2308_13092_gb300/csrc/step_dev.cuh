@@ -372,6 +372,7 @@ struct FusedStep {
   unsigned long long* imp;               // per species: impacts of this step
   int* fail;                             // first error of this step (ecpic_status)
   long long n[kMaxSpecies];              // particles before this step's births
+  int cur[kMaxSpecies];                  // buffer set of each species
   uint32_t ctr[kMaxSpecies][kNumCtr];    // counters not yet added to RunState
   uint32_t nlive;                        // particle-steps not yet added
 };
@@ -423,7 +424,9 @@ __device__ __noinline__ float3 ionize(const BatchView& b, FusedStep* fx, int s, 
   const bool ion = chk(ps >= 0 && ps < b.nseg, 18, ps, b.nseg);
   const int pspec = SP->proc[chosen].product_species;
   SegState* is = b.sst + (ion ? ps : s);
-  const int cur_e = ss->cur, cur_i = is->cur;
+  // (in k_steps the segments' own words may still be the ones from before a
+  // sort: the team's first block writes them, for the host)
+  const int cur_e = FUSED ? fx->cur[sp] : ss->cur, cur_i = FUSED ? fx->cur[ion ? pspec : sp] : is->cur;
   const long long idx_e = (FUSED ? fx->n[sp] : 0) +
                           (long long)atomicAdd(FUSED ? fx->births + sp : (unsigned long long*)&ss->n_alloc, 1ull);
   const long long idx_i =

@@ -46,7 +46,6 @@ struct StepShared {
   FusedStep fx;
   PassShared pass;
   long long cap[kMaxSpecies], fresh[kMaxSpecies];
-  int cur[kMaxSpecies];
   unsigned first[kMaxSpecies + 1];  // the team's blocks of species s: first[s] .. first[s + 1] - 1
   unsigned long long wtot[kMaxSpecies][kStepWarps];
   double owner[kFieldOwners / 8 * 9];  // eight of every nine: no bank conflicts
@@ -212,7 +211,7 @@ template <int KIND, int kStepBlock, int V>
 __device__ __forceinline__ void step_piece(int s, long long k, unsigned beg, unsigned end) {
   StepShared& sh = step_shared();
   const StepArrays a = step_arrays();
-  const PieceState ps{sh.cur[s], sh.fx.n[s], k};
+  const PieceState ps{sh.fx.cur[s], sh.fx.n[s], k};
   pass_piece<KIND, false, kStepBlock, true, V>(sh.b, &sh.run, sh.seg[s], sh.run.seg0 + s, ps, (long long)beg, (long long)end, MODE_STEP, a.dep, a.mom, a.ring, sh.pass, &sh.fx, a.E,
                                             scratch_words(sh.b.nmax, sh.spc));
 }
@@ -267,7 +266,7 @@ __device__ __noinline__ void sort_count(unsigned me, unsigned team) {
   for (int s = 0; s < ns; ++s) {
     unsigned beg, end;
     if (!step_share(sh, s, me, team, &beg, &end)) continue;
-    const int32_t* pc = sh.seg[s].cell[sh.cur[s]];
+    const int32_t* pc = sh.seg[s].cell[sh.fx.cur[s]];
     const long long n = sh.fx.n[s];
     int* h = H + s * M;
     for (unsigned q = beg + threadIdx.x; q < end; q += kStepBlock) {
@@ -320,7 +319,7 @@ __device__ __noinline__ void sort_scatter(unsigned me, unsigned team, long long*
     unsigned beg, end;
     if (!step_share(sh, s, me, team, &beg, &end)) continue;
     const SegDev& G = sh.seg[s];
-    const int a = sh.cur[s], o = a ^ 1;
+    const int a = sh.fx.cur[s], o = a ^ 1;
     const long long n = sh.fx.n[s];
     int* h = H + s * M;
     for (unsigned q = beg + tid; q < end; q += kStepBlock) {
@@ -638,7 +637,7 @@ __global__ void __launch_bounds__(kStepBlock, 1)
   if (tid < spc) {
     const SegState& q = gb.sst[(size_t)slot * spc + tid];
     sh.fx.n[tid] = q.n_proc;
-    sh.cur[tid] = q.cur;
+    sh.fx.cur[tid] = q.cur;
   }
   long long k = st->step;
   const long long step_end = st->step_end;
@@ -760,6 +759,9 @@ __global__ void __launch_bounds__(kStepBlock, 1)
       if (tid == 0) arrive(&words->arrive);
       arrivals += team;
       bool ok = await(&words->arrive, arrivals, sh);
+      // the absorbed slots end here: every block has added its own, and adds
+      // the next ones after the next barrier
+      if (ok && me == 0 && tid < ns) sst[tid].n_dead = 0;
       if (ok) {
         sort_scatter<kStepBlock>(me, team, sh.fresh);
         __syncthreads();
@@ -776,12 +778,11 @@ __global__ void __launch_bounds__(kStepBlock, 1)
         for (int c = tid + kStepBlock * (int)me; c < N; c += kStepBlock * (int)team)
           gb.hist[sh.seg[s].hoff + c] = gb.rbcnt[sh.seg[s].hoff + c] = 0;
       if (tid < ns) {
-        sh.cur[tid] ^= 1;
+        sh.fx.cur[tid] ^= 1;
         sh.fx.n[tid] = sh.fresh[tid];
         if (me == 0) {
-          sst[tid].cur = sh.cur[tid];
+          sst[tid].cur = sh.fx.cur[tid];
           sst[tid].n_proc = sst[tid].n_alloc = sst[tid].n_live = sh.fresh[tid];
-          sst[tid].n_dead = 0;
         }
       }
       __syncthreads();
