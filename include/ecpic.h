@@ -437,6 +437,12 @@ int ecpic_deposit_device2(int N, int bc, int64_t n, const int32_t* d_cell, const
  * failing check site (0 = none), out[1] = its index, out[2] = its bound,
  * out[3] = number of failed checks.  Plain builds report zeros. */
 int ecpic_debug_checks(int64_t* out4);
+/* How the last steps of a run or engine were launched: out4[0] = blocks of a
+ * launch of several steps (0: a launch per phase, or no step yet), out4[1] =
+ * threads per block, out4[2] = particles that a thread takes at a time,
+ * out4[3] = blocks of the run that has the most. */
+int ecpic_debug_route(const ecpic_run* run, int64_t* out4);
+int ecpic_engine_debug_route(const ecpic_engine* engine, int64_t* out4);
 /* Philox4x32-10 on the device: out[4i..4i+3] = Philox(counter = ctr[4i..],
  * key = key[2i..]) for i < n.  All pointers device.  Async. */
 int ecpic_philox_device(int64_t n, const uint32_t* d_ctr, const uint32_t* d_key,

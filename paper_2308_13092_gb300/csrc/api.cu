@@ -534,6 +534,13 @@ int ecpic_deposit_device2(int N, int bc, int64_t n, const int32_t* d_cell, const
   return cudaGetLastError() == cudaSuccess ? ECPIC_OK : ECPIC_ERR_CUDA;
 }
 
+int ecpic_debug_route(const ecpic_run* r, int64_t* out) {
+  if (!r || !out) return ECPIC_ERR_ARG;
+  if (!r->batch) return ECPIC_ERR_STATE;
+  r->batch->route(out);
+  return ECPIC_OK;
+}
+
 int ecpic_debug_checks(int64_t* out) {
   if (!out) return ECPIC_ERR_ARG;
   unsigned long long v[4] = {0, 0, 0, 0};

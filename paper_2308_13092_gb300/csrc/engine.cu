@@ -414,6 +414,12 @@ int ecpic_engine_sort_state(ecpic_engine* e, int* sort_every, int* since_sort) {
   return ECPIC_OK;
 }
 
+int ecpic_engine_debug_route(const ecpic_engine* e, int64_t* out) {
+  if (!e || !out) return ECPIC_ERR_ARG;
+  e->batch->route(out);
+  return ECPIC_OK;
+}
+
 int ecpic_engine_tune(ecpic_engine* e, int pass_ctas, int sort_every) {
   if (!e || pass_ctas < 0 || sort_every < 1) return ECPIC_ERR_ARG;
   e->batch->set_pass_grid(pass_ctas);

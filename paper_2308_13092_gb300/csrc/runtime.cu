@@ -1339,6 +1339,15 @@ bool Batch::several_steps() {
   return 12.0 + 3.4 * fullest_ / 512.0 < 36.0 + 11e-6 * live + 0.15 * runs && steps_fit(view(), device_);
 }
 
+void Batch::route(int64_t out[4]) const {
+  for (int i = 0; i < 4; ++i) out[i] = 0;
+  if (!took_several_) return;
+  out[0] = teams_.blocks;
+  out[1] = teams_.threads;
+  out[2] = teams_.group;
+  for (int i = 0; i < teams_.blocks; ++i) out[3] = std::max<int64_t>(out[3], teams_.size[i]);
+}
+
 int Batch::step_several(long long n, std::string* err) {
   // refused under a caller's capture, as the step graphs are: the levels and
   // sort cycles counted here would part from what the graph replays
@@ -1364,7 +1373,8 @@ int Batch::step_several(long long n, std::string* err) {
 
 int Batch::step_chunk(long long n, std::string* err) {
   cudaSetDevice(device_);
-  if (several_steps()) return step_several(n, err);
+  took_several_ = several_steps();
+  if (took_several_) return step_several(n, err);
   int rc = ensure_graphs(err);
   if (rc) return rc;
   const BatchView b = view();
@@ -1409,6 +1419,7 @@ int Batch::step_chunk(long long n, std::string* err) {
 int Batch::profile_step(long long n, double* ms, long long* launches, std::string* err) {
   cudaSetDevice(device_);
   if (pass_grid_ <= 0) pass_grid_ = choose_grid();
+  took_several_ = false;
   const BatchView b = view();
   cudaEvent_t ev[5];
   for (auto& e : ev) cudaEventCreate(&e);

@@ -122,6 +122,8 @@ class Batch {
   int phase_times(double* ms, long long* launches, long long* steps, long long* sorts,
                   std::string* err);
   int since_sort() const { return since_sort_; }
+  // how the last steps were launched (ecpic_debug_route)
+  void route(int64_t out[4]) const;
   int sort_now(std::string* err);
   // particle rebalancing of one run now, whatever its cadence (between steps)
   int rebalance_now(int slot, std::string* err);
@@ -219,6 +221,7 @@ class Batch {
   double fullest_ = 0.0;  // quads of the fullest block of teams_
   bool teams_dirty_ = true;
   StepPlan plan_{};  // of k_steps; null for a batch with more slots than blocks
+  bool took_several_ = false;  // the last chunk of steps
   std::vector<long long> level_;  // predicted level of each slot
   std::vector<long long> work_;   // its particles, as loaded or at the last growth check
   // runs admitted with defer, waiting for admit_wave()

@@ -138,6 +138,8 @@ SIGNATURES = {
     "ecpic_deposit_device2": (i32, [i32, i32, i64, vp, vp, vp, vp]),
     "ecpic_philox_device": (i32, [i64, vp, vp, vp, vp]),
     "ecpic_debug_checks": (i32, [vp]),
+    "ecpic_debug_route": (i32, [vp, vp]),
+    "ecpic_engine_debug_route": (i32, [vp, vp]),
 }
 
 _lock = threading.Lock()
@@ -165,6 +167,12 @@ def lib(build_if_missing: bool = True):
 
 def _p(a):
     return None if a is None else a.ctypes.data_as(C.c_void_p)
+
+
+def _route(out):
+    if out[0] == 0:
+        return None
+    return dict(zip(("blocks", "threads", "group", "largest_team"), out.tolist()))
 
 
 def _phase_times(call):
@@ -376,6 +384,14 @@ class Run:
         k, since = C.c_int(), C.c_int()
         _chk(self.h, self._L.ecpic_sort_state(self.h, C.byref(k), C.byref(since)), "ecpic_sort_state")
         return dict(sort_every=k.value, since_sort=since.value)
+
+    def route(self):
+        """How the last steps were launched: blocks, threads per block and
+        particles per thread of a launch of several steps, None for a launch
+        per phase (ecpic_debug_route)."""
+        out = np.zeros(4, np.int64)
+        _chk(self.h, self._L.ecpic_debug_route(self.h, _p(out)), "ecpic_debug_route")
+        return _route(out)
 
     def set_quiet_start(self, quiet=True):
         _chk(self.h, self._L.ecpic_set_quiet_start(self.h, 1 if quiet else 0),
@@ -618,6 +634,12 @@ class Engine:
         self._chk(self._L.ecpic_engine_sort_state(self.h, C.byref(k), C.byref(since)),
                   "ecpic_engine_sort_state")
         return dict(sort_every=k.value, since_sort=since.value)
+
+    def route(self):
+        """How the last steps were launched, as Run.route."""
+        out = np.zeros(4, np.int64)
+        self._chk(self._L.ecpic_engine_debug_route(self.h, _p(out)), "ecpic_engine_debug_route")
+        return _route(out)
 
     def tune(self, pass_ctas=0, sort_every=16):
         self._chk(self._L.ecpic_engine_tune(self.h, int(pass_ctas), int(sort_every)),

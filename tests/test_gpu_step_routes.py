@@ -1,0 +1,46 @@
+"""Which way a run's steps are launched (ecpic_debug_route): several steps per
+launch or a launch per phase."""
+import pytest
+
+from paper_2308_13092_gb300 import ecpic
+from helpers import gpu_from_config, require_gpu
+from test_gpu_several_steps import CASES, _ccp
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _gpu():
+    require_gpu()
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_comparison_cases_take_both_routes(case):
+    """The runs whose two routes are compared elsewhere do take them."""
+    r = gpu_from_config(CASES[case](), sort_every=16)
+    assert r.route() is None  # no step yet
+    r.step(3)
+    got = r.route()
+    assert got and got["threads"] in (256, 512) and got["blocks"] == got["largest_team"] >= 1
+    r.set_phase_timing(True)
+    r.step(3)
+    assert r.route() is None
+    r.set_phase_timing(False)
+    r.step(1)
+    assert r.route() == got
+    r.set_pass_grid(304)
+    r.step(1)
+    assert r.route() is None
+    r.sync()
+
+
+def test_engine_route():
+    e = ecpic.Engine(max_slots=4, max_cells=256, species_per_run=2)
+    for k in range(3):
+        e.submit(_ccp(128, 4000 * (k + 1), k), 40)
+    e.pump(20)
+    got = e.route()
+    assert got and got["blocks"] >= 3 and got["largest_team"] < got["blocks"]
+    e.set_phase_timing(True)
+    e.pump(10)
+    assert e.route() is None
