@@ -17,11 +17,30 @@ constexpr double kQe = 1.602176634e-19;
 constexpr double kKb = 1.380649e-23;
 constexpr size_t kAlign = 256;
 // Quads of particles per block of k_steps below which more blocks do not pay,
-// and up to which 256 threads with 255 registers beat 512 with 128 (us per
-// step, without samples and sorts: 12.1 against 13.6 with 96 quads per block,
-// 20.6 against 20.4 with 431, 26.1 against 23.7 with 862).
+// and up to which 256 threads with 255 registers beat 512 with 128: one
+// iteration of them (us per step, samples every 20 steps, 256 : 512 threads:
+// 10.6 : 12.0 with 96 quads per block, 11.1 : 11.8 with 216, 13.3 : 12.0 with
+// 291, 14.3 : 13.3 with 431).
 constexpr double kStepQuads = 48.0;
-constexpr double kStepSmall = 400.0;
+constexpr double kStepSmall = 256.0;
+// The share of the SMs that a run's blocks may take.  A block of k_steps has
+// its SM to itself, so a small run that took them all would keep out the runs
+// of other streams for little: it gets a quarter or a third while a block then
+// has one iteration of 512 threads, and half up to 1.5 of them.  us per step of
+// all of 1 / 4 / 8 / 16 such runs at once, launch per phase : every SM : share:
+// 16,384 particles 28, 30, 32, 52 : 10, 40, 80, 160 : 11, 11, 21, 42 (quarter);
+// 58,254 27, 32, 39, 71 : 11, 42, 83, 167 : 12, 12, 25, 49 (quarter); 100,000
+// 31, 38, 55, 107 : 13, 48, 97, 194 : 13, 20, 37, 73 (third); 131,072 30, 41, 69,
+// 137 : 13, 49, 98, 197 : 13, 27, 53, 106 (half); 220,000 32, 52, 101, 198 : 13,
+// 53, 106, 212 : 16, 32, 64, 129 (half).  262,144 take all: 32, 59, 110, 219 : 14,
+// 54, 108, 217.
+int step_share_of(double work, int sms) {
+  const double q = work / 4.0;
+  if (q <= 512.0 * (sms / 4)) return std::max(1, sms / 4);
+  if (q <= 512.0 * (sms / 3)) return std::max(1, sms / 3);
+  if (q <= 768.0 * (sms / 2)) return std::max(1, sms / 2);
+  return sms;
+}
 // Particles of the fullest block up to which a thread takes one or two of them
 // at a time instead of four: a block's time is then the chain of one warp's
 // instructions, which are fewer (us per step: 16,384 particles, 195 per block,
@@ -1281,8 +1300,9 @@ int Batch::step(long long n, std::string* err) {
 }
 
 // The blocks of k_steps among the resident runs: one each, the others where
-// the most particles per block are, down to kStepQuads quads per block.
-// Formed again when the runs or their sizes changed.
+// the most particles per block are, down to kStepQuads quads per block and up
+// to a run's share of the SMs.  Formed again when the runs or their sizes
+// changed.
 void Batch::form_teams() {
   if (!teams_dirty_) return;
   teams_dirty_ = false;
@@ -1298,7 +1318,7 @@ void Batch::form_teams() {
     double top = 4.0 * kStepQuads;
     for (size_t i = 0; i < slots.size(); ++i) {
       const double per = (double)work_[slots[i]] / size[i];
-      if (per > top) {
+      if (per > top && size[i] < step_share_of((double)work_[slots[i]], most)) {
         top = per;
         best = (int)i;
       }

@@ -44,3 +44,21 @@ def test_engine_route():
     e.set_phase_timing(True)
     e.pump(10)
     assert e.route() is None
+
+
+@pytest.mark.parametrize("n,parts,threads", [
+    (600, 4, 256), (8192, 4, 256), (29127, 4, 512), (50000, 3, 512), (65536, 2, 512), (110000, 2, 512),
+    (131072, 1, 512),
+])
+def test_a_small_run_leaves_room_for_others(n, parts, threads):
+    """A block of several steps per launch has its SM to itself, so a run that
+    cannot use them all takes a share, and runs on other streams the rest."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    r = gpu_from_config(_ccp(128, n, 3))
+    r.step(2)
+    got = r.route()
+    assert got and got["threads"] == threads and got["blocks"] <= sms // parts, got
+    if parts < 4:  # and no less than it needs
+        assert got["blocks"] > sms // (parts + 1), got
+    r.sync()
