@@ -1340,12 +1340,15 @@ void Batch::form_teams() {
 }
 
 // Whether the batch advances by k_steps.  Its step takes the time of its
-// fullest block, 12 us + 3.4 us per 512 quads; a step of one launch per phase
-// takes 36 us + 11 us per million particles + 0.15 us per run.  Measured, both
-// ways, us per step: one run of 0.5 / 2.1 / 8.4 million particles 18.5 / 35 /
-// 107 against 36 / 61 / 125; 16 runs of 2.5 million 44 against 65; 64 runs of
-// 1.3 / 3.9 / 13 million 38 / 90 / 275 against 62 / 95 / 188; 140 runs of 2.6
-// million, the largest on one block, 109 against 86.
+// fullest block, 12 us + 3.45 us per 512 quads; a step of one launch per phase
+// takes 36 us + 9.3 us per million particles + 0.17 us per run.  Measured, both
+// ways (k_steps : launch per phase), us per step with samples every 20 or 40
+// steps and sorts every 32.  One run of 0.5 / 2.1 / 4.2 / 8.4 million particles
+// 18 : 38, 38 : 62, 61 : 79, 108 : 116; of 16.8 / 50 million 201 : 185 and 566 :
+// 495 on 1024 cells, 207 : 204 and 625 : 513 on 2048.  Batches: 16 runs of 3.9 /
+// 11.8 million in all 59 : 80, 151 : 157; 32 of 2.3 / 7.5 million 38 : 60, 112 :
+// 113; 64 of 1.5 / 4.5 / 15 million 33 : 60, 77 : 93, 232 : 185; 140 of 3.3 / 9.8
+// million, the largest on two blocks, 106 : 93, 302 : 155.
 bool Batch::several_steps() {
   if (!use_graphs_ || timing_ || pass_grid_override_ != 0 || !plan_.words) return false;
   form_teams();
@@ -1356,7 +1359,7 @@ bool Batch::several_steps() {
       runs += 1.0;
     }
   if (runs == 0.0) return false;
-  return 12.0 + 3.4 * fullest_ / 512.0 < 36.0 + 11e-6 * live + 0.15 * runs && steps_fit(view(), device_);
+  return 12.0 + 3.45 * fullest_ / 512.0 < 36.0 + 9.3e-6 * live + 0.17 * runs && steps_fit(view(), device_);
 }
 
 void Batch::route(int64_t out[4]) const {

@@ -62,3 +62,13 @@ def test_a_small_run_leaves_room_for_others(n, parts, threads):
     if parts < 4:  # and no less than it needs
         assert got["blocks"] > sms // (parts + 1), got
     r.sync()
+
+
+@pytest.mark.parametrize("million,several", [(2.0, True), (8.0, True), (20.0, False)])
+def test_a_large_run_takes_a_launch_per_phase(million, several):
+    """Beyond some 13 million particles of one run its blocks of several steps
+    per launch have too few warps against the phase kernels'."""
+    r = gpu_from_config(_ccp(1024, int(million * 5e5), 3, L=0.3))
+    r.step(2)
+    assert (r.route() is not None) == several
+    r.sync()
