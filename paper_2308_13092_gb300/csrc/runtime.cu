@@ -1193,7 +1193,10 @@ int Batch::rb_first_due(int steps) const {
 
 void Batch::advance_levels(int steps) {
   for (int s = 0; s < max_slots_; ++s)
-    if (active_[s]) level_[s] = std::min(level_[s] + steps, specs_[s].step_end);
+    if (advances(s)) {
+      level_[s] = std::min(level_[s] + steps, specs_[s].step_end);
+      if (!advances(s)) teams_dirty_ = true;  // its blocks go to the others
+    }
 }
 
 void Batch::rebalance_launch() {
@@ -1299,10 +1302,10 @@ int Batch::step(long long n, std::string* err) {
   return ECPIC_OK;
 }
 
-// The blocks of k_steps among the resident runs: one each, the others where
-// the most particles per block are, down to kStepQuads quads per block and up
-// to a run's share of the SMs.  Formed again when the runs or their sizes
-// changed.
+// The blocks of k_steps among the resident runs that are not at their end: one
+// each, the others where the most particles per block are, down to kStepQuads
+// quads per block and up to a run's share of the SMs.  Formed again when the
+// runs or their sizes changed.
 void Batch::form_teams() {
   if (!teams_dirty_) return;
   teams_dirty_ = false;
@@ -1311,7 +1314,7 @@ void Batch::form_teams() {
   const int most = std::min(sm_count_, kMaxStepBlocks);
   std::vector<int> slots, size;
   for (int s = 0; s < max_slots_; ++s)
-    if (active_[s]) slots.push_back(s);
+    if (advances(s)) slots.push_back(s);
   size.assign(slots.size(), 1);
   for (int used = (int)slots.size(); used < most; ++used) {
     int best = -1;
@@ -1354,7 +1357,7 @@ bool Batch::several_steps() {
   form_teams();
   double live = 0.0, runs = 0.0;
   for (int s = 0; s < max_slots_; ++s)
-    if (active_[s]) {
+    if (advances(s)) {
       live += (double)work_[s];
       runs += 1.0;
     }
@@ -1881,6 +1884,7 @@ int Batch::set_step_end(int slot, long long step_end, std::string* err) {
   st.step_end = step_end;
   specs_[slot].step_end = step_end;
   level_[slot] = std::min<long long>(st.step, step_end);
+  teams_dirty_ = true;
   return check(cudaMemcpy(d_rst_ + slot, &st, sizeof(RunState), cudaMemcpyHostToDevice),
                "set_step_end", err);
 }

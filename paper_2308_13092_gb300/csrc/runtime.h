@@ -171,6 +171,8 @@ class Batch {
   int choose_grid() const;
   bool stage_field(int grid) const;
   int step_chunk(long long n, std::string* err);
+  // a resident run that has not reached its end
+  bool advances(int s) const { return active_[s] && level_[s] < specs_[s].step_end; }
   bool several_steps();
   void form_teams();
   size_t plan_deposit_bytes() const { return 2 * sizeof(unsigned long long) * (size_t)spc_ * (size_t)(nmax_ + 1); }

@@ -72,3 +72,19 @@ def test_a_large_run_takes_a_launch_per_phase(million, several):
     r.step(2)
     assert (r.route() is not None) == several
     r.sync()
+
+
+def test_runs_at_their_end_hold_no_blocks():
+    """A finished run that is still resident leaves its blocks to the others:
+    here within one pump, whose steps go in chunks of at most 64."""
+    e = ecpic.Engine(max_slots=2, max_cells=256, species_per_run=2)
+    t = [e.submit(_ccp(128, 200000, 1), 200), e.submit(_ccp(128, 262144, 2), 10)]
+    e.pump(5)
+    both = e.route()
+    assert both and both["largest_team"] < both["blocks"]
+    e.pump(150)
+    alone = e.route()
+    assert alone and alone["largest_team"] == alone["blocks"] == both["blocks"]
+    while sum(e.pump(64)):
+        pass
+    assert [e.poll(k, diagnostics=True)["diag"]["step"] for k in t] == [200, 10]
