@@ -1737,8 +1737,9 @@ int Batch::set_particles(int slot, int species, const int32_t* cell, const float
   cudaSetDevice(device_);
   int rc = check(cudaStreamSynchronize(stream_), "synchronize", err);
   if (rc) return rc;
-  SegState ss;
-  cudaMemcpy(&ss, d_sst_ + seg, sizeof(SegState), cudaMemcpyDeviceToHost);
+  std::vector<SegState> all(spc_);  // the run's
+  cudaMemcpy(all.data(), d_sst_ + slot * spc_, sizeof(SegState) * spc_, cudaMemcpyDeviceToHost);
+  SegState& ss = all[species];
   const int u = ss.cur;
   const size_t m = (size_t)n;
   cudaMemcpy(G.cell[u], cell, 4 * m, cudaMemcpyHostToDevice);
@@ -1754,6 +1755,9 @@ int Batch::set_particles(int slot, int species, const int32_t* cell, const float
   ss.n_proc = ss.n_alloc = n;
   ss.n_dead = 0;
   cudaMemcpy(d_sst_ + seg, &ss, sizeof(SegState), cudaMemcpyHostToDevice);
+  work_[slot] = 0;
+  for (const SegState& q : all) work_[slot] += q.n_alloc;
+  teams_dirty_ = true;
   refresh(slot);
   return check(cudaGetLastError(), "set_particles", err);
 }

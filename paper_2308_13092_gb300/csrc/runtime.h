@@ -225,7 +225,7 @@ class Batch {
   StepPlan plan_{};  // of k_steps; null for a batch with more slots than blocks
   bool took_several_ = false;  // the last chunk of steps
   std::vector<long long> level_;  // predicted level of each slot
-  std::vector<long long> work_;   // its particles, as loaded or at the last growth check
+  std::vector<long long> work_;   // its particles, as loaded, set or at the last growth check
   // runs admitted with defer, waiting for admit_wave()
   std::vector<int> wave_slots_;
   std::vector<InitParams> wave_params_;

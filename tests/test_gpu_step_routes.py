@@ -88,3 +88,23 @@ def test_runs_at_their_end_hold_no_blocks():
     while sum(e.pump(64)):
         pass
     assert [e.poll(k, diagnostics=True)["diag"]["step"] for k in t] == [200, 10]
+
+
+def test_a_run_filled_by_its_caller_gets_its_blocks():
+    """Sizes follow set_particles: a run that starts with few particles and is
+    filled afterwards gets the blocks of its new size."""
+    import numpy as np
+    c = _ccp(128, 64, 3)
+    for s in c.species:
+        s.capacity = 200000
+    r = gpu_from_config(c)
+    r.step(1)
+    assert r.route()["blocks"] == 1
+    n = 150000
+    rng = np.random.default_rng(1)
+    for s in range(2):
+        v = rng.normal(0.0, 1e3, (3, n)).astype(np.float32)
+        r.set_particles(s, rng.integers(0, 128, n), rng.random(n, np.float32) * np.float32(0.99), *v, np.arange(n))
+    r.step(1)
+    r.sync()
+    assert r.route()["blocks"] >= 128 and r.route()["threads"] == 512
