@@ -443,6 +443,10 @@ int ecpic_debug_checks(int64_t* out4);
  * out4[3] = blocks of the run that has the most. */
 int ecpic_debug_route(const ecpic_run* run, int64_t* out4);
 int ecpic_engine_debug_route(const ecpic_engine* engine, int64_t* out4);
+/* Blocks that a launch of several steps may have (0: one per SM).  More than
+ * the device holds at once make it refuse the launch, as it does on a stream
+ * with a part of the SMs: the run then takes a launch per phase. */
+int ecpic_debug_step_blocks(ecpic_run* run, int blocks);
 /* Philox4x32-10 on the device: out[4i..4i+3] = Philox(counter = ctr[4i..],
  * key = key[2i..]) for i < n.  All pointers device.  Async. */
 int ecpic_philox_device(int64_t n, const uint32_t* d_ctr, const uint32_t* d_key,

@@ -541,6 +541,13 @@ int ecpic_debug_route(const ecpic_run* r, int64_t* out) {
   return ECPIC_OK;
 }
 
+int ecpic_debug_step_blocks(ecpic_run* r, int blocks) {
+  if (!r || blocks < 0) return ECPIC_ERR_ARG;
+  if (!r->batch) return fail(r, ECPIC_ERR_STATE, "init first");
+  r->batch->set_step_blocks(blocks);
+  return ECPIC_OK;
+}
+
 int ecpic_debug_checks(int64_t* out) {
   if (!out) return ECPIC_ERR_ARG;
   unsigned long long v[4] = {0, 0, 0, 0};

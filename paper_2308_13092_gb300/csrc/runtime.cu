@@ -1311,7 +1311,7 @@ void Batch::form_teams() {
   teams_dirty_ = false;
   teams_ = StepTeams{};
   fullest_ = 0.0;
-  const int most = std::min(sm_count_, kMaxStepBlocks);
+  const int most = std::min(step_blocks_ > 0 ? step_blocks_ : sm_count_, kMaxStepBlocks);
   std::vector<int> slots, size;
   for (int s = 0; s < max_slots_; ++s)
     if (advances(s)) slots.push_back(s);
@@ -1353,7 +1353,7 @@ void Batch::form_teams() {
 // 113; 64 of 1.5 / 4.5 / 15 million 33 : 60, 77 : 93, 232 : 185; 140 of 3.3 / 9.8
 // million, the largest on two blocks, 106 : 93, 302 : 155.
 bool Batch::several_steps() {
-  if (!use_graphs_ || timing_ || pass_grid_override_ != 0 || !plan_.words) return false;
+  if (!use_graphs_ || timing_ || pass_grid_override_ != 0 || no_several_ || !plan_.words) return false;
   form_teams();
   double live = 0.0, runs = 0.0;
   for (int s = 0; s < max_slots_; ++s)
@@ -1385,7 +1385,15 @@ int Batch::step_several(long long n, std::string* err) {
   const BatchView b = view();
   while (n > 0) {
     const int m = rb_first_due((int)std::min<long long>(n, kStepsPerLaunch));
-    int rc = check(launch_steps(b, plan_, teams_, m, sort_every_, since_sort_, stream_), "steps", err);
+    const cudaError_t e = launch_steps(b, plan_, teams_, m, sort_every_, since_sort_, stream_);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+      // the blocks cannot all be resident (a stream with a part of the SMs):
+      // nothing was launched, and this batch takes a launch per phase from here
+      cudaGetLastError();
+      no_several_ = true;
+      return step_chunk(n, err);
+    }
+    int rc = check(e, "steps", err);
     if (rc) return rc;
     n -= m;
     since_sort_ = (since_sort_ + m) % sort_every_;

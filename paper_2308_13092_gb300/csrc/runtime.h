@@ -124,6 +124,7 @@ class Batch {
   int since_sort() const { return since_sort_; }
   // how the last steps were launched (ecpic_debug_route)
   void route(int64_t out[4]) const;
+  void set_step_blocks(int n) { step_blocks_ = n; teams_dirty_ = true; }
   int sort_now(std::string* err);
   // particle rebalancing of one run now, whatever its cadence (between steps)
   int rebalance_now(int slot, std::string* err);
@@ -224,6 +225,8 @@ class Batch {
   bool teams_dirty_ = true;
   StepPlan plan_{};  // of k_steps; null for a batch with more slots than blocks
   bool took_several_ = false;  // the last chunk of steps
+  bool no_several_ = false;    // its launch was refused once
+  int step_blocks_ = 0;        // blocks of k_steps at most (0: one per SM)
   std::vector<long long> level_;  // predicted level of each slot
   std::vector<long long> work_;   // its particles, as loaded, set or at the last growth check
   // runs admitted with defer, waiting for admit_wave()

@@ -140,6 +140,7 @@ SIGNATURES = {
     "ecpic_debug_checks": (i32, [vp]),
     "ecpic_debug_route": (i32, [vp, vp]),
     "ecpic_engine_debug_route": (i32, [vp, vp]),
+    "ecpic_debug_step_blocks": (i32, [vp, i32]),
 }
 
 _lock = threading.Lock()
@@ -392,6 +393,9 @@ class Run:
         out = np.zeros(4, np.int64)
         _chk(self.h, self._L.ecpic_debug_route(self.h, _p(out)), "ecpic_debug_route")
         return _route(out)
+
+    def debug_step_blocks(self, blocks):
+        _chk(self.h, self._L.ecpic_debug_step_blocks(self.h, int(blocks)), "ecpic_debug_step_blocks")
 
     def set_quiet_start(self, quiet=True):
         _chk(self.h, self._L.ecpic_set_quiet_start(self.h, 1 if quiet else 0),

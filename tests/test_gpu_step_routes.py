@@ -4,7 +4,7 @@ import pytest
 
 from paper_2308_13092_gb300 import ecpic
 from helpers import gpu_from_config, require_gpu
-from test_gpu_several_steps import CASES, _ccp
+from test_gpu_several_steps import CASES, _ccp, _state
 
 pytestmark = pytest.mark.gpu
 
@@ -108,3 +108,30 @@ def test_a_run_filled_by_its_caller_gets_its_blocks():
     r.step(1)
     r.sync()
     assert r.route()["blocks"] >= 128 and r.route()["threads"] == 512
+
+
+def test_refused_launch_takes_a_launch_per_phase():
+    """More blocks than the device holds at once: the cooperative launch is
+    refused on the host, nothing runs, and the steps go a launch per phase."""
+    import numpy as np
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms >= 160:
+        pytest.skip("a launch has at most 160 blocks")
+    a, b = (gpu_from_config(_ccp(128, 150000, 3), sort_every=16) for _ in range(2))
+    for r in (a, b):
+        r.step(5)
+        assert r.route()["blocks"] == sms
+    a.debug_step_blocks(160)
+    a.step(30)
+    assert a.route() is None
+    b.step(30)
+    a.sync()
+    b.sync()
+    assert a.diagnostics()["species"] == b.diagnostics()["species"]
+    for x, y in zip(_state(a)[2], _state(b)[2]):
+        assert all(np.array_equal(u, v) for u, v in zip(x, y))
+    a.debug_step_blocks(0)  # once refused, it stays a launch per phase
+    a.step(1)
+    assert a.route() is None
+    a.sync()
