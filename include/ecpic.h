@@ -216,8 +216,9 @@ int ecpic_set_tallies(ecpic_run* run, double eedf_center_m, double eedf_halfwidt
 int ecpic_init(ecpic_run* run, uint64_t seed, double dt_s,
                const int64_t* n_per_species, const double* T_eV);
 /* Advance n_steps (async; a run or batch that does not fill the device takes
- * several steps per launch, others replay a graph of launches).  One step: EC (or MC) gather and leapfrog push
- * (Eq. 6-9), wall absorption, null-collision MCC, CIC deposit (Eq. 2-3),
+ * several steps per launch, others replay a graph of launches; with automatic
+ * growth the host reads the sizes about every 64 steps).  One step: EC (or MC)
+ * gather and leapfrog push (Eq. 6-9), wall absorption, null-collision MCC, CIC deposit (Eq. 2-3),
  * Poisson (Eq. 4) and field (Eq. 5) of the next time level. */
 int ecpic_step(ecpic_run* run, int64_t n_steps);
 /* Wait for queued work; return the first device-side error of the run. */
@@ -293,7 +294,9 @@ int ecpic_autotune_ks(ecpic_run* run, int64_t steps_per_trial, const int* ks, in
  * phases (CUDA events on the run's stream) to running sums.  The sums thus
  * come from the very replays that advance the run, not from a separate
  * profiling pass.  While it is on, a run that would take several steps per
- * launch takes a launch per phase instead, with the same results.  on = 0 restores the plain graphs (the sums are kept). */
+ * launch takes a launch per phase instead: the same trajectory, sampled sums
+ * equal to FP32 rounding.  on = 0 restores the plain graphs (the sums are
+ * kept). */
 int ecpic_set_phase_timing(ecpic_run* run, int on);
 /* Read and clear the phase sums (waits for the timed steps): ms[0..3] = the
  * particle pass, the field solve, the counting sort, the real-collision

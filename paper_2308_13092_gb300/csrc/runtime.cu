@@ -47,7 +47,8 @@ int step_share_of(double work, int sms) {
 // 12.2 with one, 12.7 with two, 13.1 with four; 58,254, 383 per block, 12.7,
 // 12.2 and 13.3; 131,072, 862 per block, 13.8 with two, 13.2 with four).
 constexpr double kStepOne = 256.0, kStepTwo = 512.0;
-// Steps of one launch of k_steps (a launch costs about 10 us).
+// Steps of one launch of k_steps at most (a launch costs about 10 us; with
+// automatic growth the sizes are read every 64 steps or sort cycle).
 constexpr long long kStepsPerLaunch = 256;
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }

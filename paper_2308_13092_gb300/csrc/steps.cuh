@@ -3,8 +3,8 @@
 // A batch that does not fill the device is bound by latency, not by bytes: a
 // step of three dependent launches (k_pass, k_collide, k_field) spends its
 // time in their prologues, drains and hand-overs (a run of 16,384 particles:
-// 31 us per step for 0.1 us of traffic).  k_steps keeps one block per SM for a
-// run of steps.  Every block belongs to one run (its team shares the run's
+// 28 us per step for 0.1 us of traffic).  k_steps keeps a block on each of its
+// SMs for a run of steps.  Every block belongs to one run (its team shares the run's
 // particles); the run's tables, grid and field stay in shared memory, real
 // collisions are carried out by the pass itself (a thread has two or four
 // times the pass kernel's registers), and each block solves the run's field
@@ -13,11 +13,10 @@
 // one another.  A sample step adds its sums in shared memory as fixed-point
 // integers (mom_add4) and shares its moments among the team's blocks.
 //
-// Measured, us per step with samples every 10-20 steps and sorts every 16-32
-// (one launch per phase : here): 16,384 particles on 128 cells 31.4 : 12.2;
-// 58,254 on 114 doubling cells 30.6 : 12.2; 524,288 on 1024 cells 40.5 : 18.9;
-// 2.1 million on 2048 cells 70.5 : 39; 12 periodic runs of 131,072 on 2048
-// cells 44.8 : 23.6.  What is left of the smallest step: the chain of a piece
+// Measured, us per step of one run with samples every 20 steps and sorts every
+// 32 (one launch per phase : here): 16,384 particles on 128 cells 28 : 11; 58,254
+// on 114 cells 27 : 12; 524,288 on 1024 cells 38 : 18; 2.1 million on 2048 cells
+// 62 : 37.  What is left of the smallest step: the chain of a piece
 // (loads, Philox, push, deposit, null-collision test, flush), the barrier and
 // the field, about 6, 2 and 4 us.
 //
