@@ -1362,7 +1362,7 @@ bool Batch::several_steps() {
       live += (double)work_[s];
       runs += 1.0;
     }
-  if (runs == 0.0) return false;
+  if (runs == 0.0) return true;  // (every run is at its end: no launch)
   return 12.0 + 3.45 * fullest_ / 512.0 < 36.0 + 9.3e-6 * live + 0.17 * runs && steps_fit(view(), device_);
 }
 
@@ -1386,7 +1386,8 @@ int Batch::step_several(long long n, std::string* err) {
   const BatchView b = view();
   while (n > 0) {
     const int m = rb_first_due((int)std::min<long long>(n, kStepsPerLaunch));
-    const cudaError_t e = launch_steps(b, plan_, teams_, m, sort_every_, since_sort_, stream_);
+    const cudaError_t e = teams_.blocks == 0 ? cudaSuccess
+                                             : launch_steps(b, plan_, teams_, m, sort_every_, since_sort_, stream_);
     if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
       // the blocks cannot all be resident (a stream with a part of the SMs):
       // nothing was launched, and this batch takes a launch per phase from here

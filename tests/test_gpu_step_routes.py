@@ -135,3 +135,21 @@ def test_refused_launch_takes_a_launch_per_phase():
     a.step(1)
     assert a.route() is None
     a.sync()
+
+
+def test_steps_past_the_end_of_every_run():
+    """A pump for more steps than any run has left: nothing is launched for the
+    rest, and the runs end as they do one pump at a time."""
+    import numpy as np
+    out = []
+    for pumps in ((10, 400), (10, 10, 10, 10)):
+        e = ecpic.Engine(max_slots=2, max_cells=256, species_per_run=2)
+        t = [e.submit(_ccp(128, 4000, 1), 40), e.submit(_ccp(100, 3000, 2), 20)]
+        for n in pumps:
+            left = e.pump(n)
+        assert left == (0, 0)
+        out.append([e.poll(k, diagnostics=True, profiles=True)["diag"] for k in t])
+    assert [d["step"] for d in out[0]] == [40, 20]
+    for a, b in zip(*out):
+        assert a["species"] == b["species"] and a["n_samples"] == b["n_samples"]
+        assert np.array_equal(a["density"], b["density"])
